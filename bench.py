@@ -109,7 +109,7 @@ def device_roofs(dev, sm_mhz):
                       "during the timed steps)"}
 
 
-KERNEL_SOURCES = ("mocca.cu", "osscir_internal.cuh", "osscir_launch.h")
+KERNEL_SOURCES = ("mocca.cu", "osscir_dfl.cuh", "osscir_internal.cuh", "osscir_launch.h")
 
 
 def _source_sha() -> str:

@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libosscir.so")
 SOURCES = ["batch.cu", "capi.cu", "geometry.cu", "mocca.cu", "noalloc.cu", "noise.cu", "server.cu"]
-HEADERS = ["osscir_internal.cuh", "osscir_launch.h", "osscir_ctx.h"]
+HEADERS = ["osscir_dfl.cuh", "osscir_internal.cuh", "osscir_launch.h", "osscir_ctx.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: no implicit contraction of a * b + c.  Every fused multiply-add
 # is an explicit fmaf / fma in the source, so each kernel computes the same
