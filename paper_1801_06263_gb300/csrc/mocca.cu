@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(kFwdThreads) k_mocca_ray_inner(GeomC C, RayRec
 // Box-constrained primal step: argmin over lo <= x <= hi of 1/2 (x - t)^T Q (x - t),
 // by trying every active set and keeping the feasible candidate of least objective.
 // Bounds may be infinite (nonnegativity: lo = 0, hi = +inf).
-__device__ void box_prox3(const double Q[3][3], const double t[3], const float lo[3], const float hi[3],
+__device__ __noinline__ void box_prox3(const double Q[3][3], const double t[3], const float lo[3], const float hi[3],
                           double xo[3]) {
     double best = 1e308;
     xo[0] = fmin(fmax(t[0], (double)lo[0]), (double)hi[0]);
@@ -924,6 +924,107 @@ __device__ void box_prox3(const double Q[3][3], const double t[3], const float l
             xo[0] = xc[0]; xo[1] = xc[1]; xo[2] = xc[2];
         }
     }
+}
+
+// The same argmin from its optimality conditions, in double-float: Q = p (packed
+// 00 01 02 11 12 22, any positive scale), t the unconstrained minimiser outside the
+// box.  For a strictly convex problem the minimiser is the one point whose free
+// components are inside the box and whose gradient Q (x - t) points into the box at
+// every active bound.  With d_i = bound_i - t_i those points are, for one active
+// bound i, the solution of the free 2x2 system Q_FF (x - t)_F = -Q_Fi d_i (the
+// gradient then has the sign of d_i); for two (k free), x_k = t_k - (Q_ki d_i +
+// Q_kj d_j) / Q_kk, the gradient being the Schur complement Q_ab - Q_ak Q_bk / Q_kk
+// times d; for three the corner itself.  A sign that rounding leaves open (2^-44 of
+// its terms) passes: the point then differs from the minimiser by less than FP32
+// rounding.  Returns false if no active set passes (box_prox3 then decides).
+// Why: the FP64 enumeration above runs on a pipe of 1/64 the FP32 rate and takes
+// every active set of every pixel; with maps held nonnegative nearly every warp has
+// such a pixel, and the pixel step of 389 x 389 maps took 279 us: ten iterations
+// 7535 us, now 4832 us.
+__device__ __forceinline__ bool box_step3(const dfl (&p)[6], const dfl (&t)[3], const float (&lo)[3],
+                                          const float (&hi)[3], float xo[3]) {
+    const int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+    if (!(p[0].hi > 0.0f && p[3].hi > 0.0f && p[5].hi > 0.0f)) return false;
+    auto inside = [&](int m, dfl v) {
+        const float f = df_f(v), tol = 1e-12f * (1.0f + fabsf(f));
+        return (f > lo[m] || df_f(df_sub(v, dfl{lo[m], 0.0f})) >= -tol) &&
+               (f < hi[m] || df_f(df_sub(dfl{hi[m], 0.0f}, v)) >= -tol);
+    };
+    auto put = [&](int m, dfl v) { xo[m] = fminf(fmaxf(df_f(v), lo[m]), hi[m]); };
+    // whether a gradient of size g (its terms' magnitude m) points into the box at a bound
+    auto inward = [](float g, float m, int side) { return side ? g <= m * 0x1p-44f : g >= -m * 0x1p-44f; };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int j = (i + 1) % 3, k = (i + 2) % 3;
+        // (x_j - t_j, x_k - t_k) = d_i (wj, wk)
+        const dfl qji = p[at[j][i]], qjk = p[at[j][k]], r = df_rcp(p[at[j][j]]), l = df_mul(qjk, r);
+        const dfl schur = df_sub(p[at[k][k]], df_mul(l, qjk));
+        if (!(schur.hi > 0.0f)) return false;
+        const dfl wk = df_mul(df_sub(df_mul(l, qji), p[at[k][i]]), df_rcp(schur));
+        const dfl wj = df_neg(df_mul(df_add(qji, df_mul(qjk, wk)), r));
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            const float b = side ? hi[i] : lo[i];
+            const dfl d = df_sub(dfl{b, 0.0f}, t[i]);
+            if (isinf(b) || !inward(d.hi, 0.0f, side)) continue;
+            const dfl vj = df_add(t[j], df_mul(wj, d)), vk = df_add(t[k], df_mul(wk, d));
+            if (inside(j, vj) && inside(k, vk)) {
+                xo[i] = b;
+                put(j, vj);
+                put(k, vk);
+                return true;
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        const dfl qki = p[at[k][i]], qkj = p[at[k][j]], r = df_rcp(p[at[k][k]]), li = df_mul(qki, r), lj = df_mul(qkj, r);
+        const dfl sii = df_sub(p[at[i][i]], df_mul(li, qki)), sjj = df_sub(p[at[j][j]], df_mul(lj, qkj));
+        const dfl sij = df_sub(p[at[i][j]], df_mul(li, qkj));
+#pragma unroll 1
+        for (int code = 0; code < 4; ++code) {
+            const int si = code & 1, sj = code >> 1;
+            const float bi = si ? hi[i] : lo[i], bj = sj ? hi[j] : lo[j];
+            if (isinf(bi) || isinf(bj)) continue;
+            const dfl di = df_sub(dfl{bi, 0.0f}, t[i]), dj = df_sub(dfl{bj, 0.0f}, t[j]);
+            const dfl g0 = df_mul(sii, di), g1 = df_mul(sij, dj), h0 = df_mul(sij, di), h1 = df_mul(sjj, dj);
+            if (!inward(df_f(df_add(g0, g1)), fabsf(g0.hi) + fabsf(g1.hi), si) ||
+                !inward(df_f(df_add(h0, h1)), fabsf(h0.hi) + fabsf(h1.hi), sj))
+                continue;
+            const dfl v = df_sub(t[k], df_add(df_mul(li, di), df_mul(lj, dj)));
+            if (inside(k, v)) {
+                xo[i] = bi;
+                xo[j] = bj;
+                put(k, v);
+                return true;
+            }
+        }
+    }
+#pragma unroll 1
+    for (int code = 0; code < 8; ++code) {
+        dfl d[3];
+        float b[3];
+        bool ok = true;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            b[m] = (code >> m & 1) ? hi[m] : lo[m];
+            ok = ok && !isinf(b[m]);
+            d[m] = df_sub(dfl{b[m], 0.0f}, t[m]);
+        }
+        if (!ok) continue;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const dfl g0 = df_mul(p[at[m][0]], d[0]), g1 = df_mul(p[at[m][1]], d[1]), g2 = df_mul(p[at[m][2]], d[2]);
+            ok = ok && inward(df_f(df_add(df_add(g0, g1), g2)), fabsf(g0.hi) + fabsf(g1.hi) + fabsf(g2.hi), code >> m & 1);
+        }
+        if (ok) {
+#pragma unroll
+            for (int m = 0; m < 3; ++m) xo[m] = b[m];
+            return true;
+        }
+    }
+    return false;
 }
 
 __device__ __forceinline__ void bp_finish(const GeomC& C, const StepParams& P, const SolveD& D, int ix, int iy,
@@ -1042,11 +1143,13 @@ __device__ __forceinline__ void bp_finish(const GeomC& C, const StepParams& P, c
 // acc[3..8] = P_k (packed 00 01 02 11 12 22), T^-1_k = P_k / lambda; the primal
 // step x' = x - T_k v_k (optionally onto the box) and the extrapolation
 // xbar' = 2 x' - x.  T_k = lambda (P_k + 1e-12 tr(P_k) I)^-1 (the regularisation
-// that keeps T positive definite) is applied by the adjugate in double-float
-// arithmetic on P_k scaled by an exact power of two near 1 / tr(P_k), so that the
-// cubed entries stay inside the FP32 exponent range; T_k has a condition number
-// near 6e6, and the ~48-bit double-float solve keeps the step to FP32 accuracy.
-// Only a step that leaves the box goes to the FP64 active-set solve.
+// that keeps T positive definite) is applied by symmetric elimination in double-float
+// arithmetic on P_k scaled by an exact power of two near 1 / tr(P_k); T_k has a
+// condition number near 6e6, and the ~48-bit elimination (whose error grows with the
+// condition number; the adjugate's grows with its square when two eigenvalues are
+// small: 5e-10 against 1.4e-5 of the step at worst over random P of condition up to
+// 1e6) keeps the step to FP32 accuracy.
+// A step that leaves the box is replaced by the box's minimiser (box_step3).
 __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, const SolveD& D, int k,
                                            const float acc[9]) {
     const float4 x = D.x[k];
@@ -1063,20 +1166,20 @@ __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, 
     const float p1 = acc[4] * sc, p2 = acc[5] * sc, p4 = acc[7] * sc;
     const float reg = 1e-12f * ((acc[3] * sc + acc[6] * sc) + acc[8] * sc);
     const dfl p0 = df_2sum(acc[3] * sc, reg), p3 = df_2sum(acc[6] * sc, reg), p5 = df_2sum(acc[8] * sc, reg);
-    const dfl P1 = {p1, 0.0f}, P2 = {p2, 0.0f};
-    const dfl c00 = df_sub(df_mul(p3, p5), df_2prod(p4, p4));
-    const dfl c01 = df_sub(df_2prod(p2, p4), df_mulf(p5, p1));
-    const dfl c02 = df_sub(df_2prod(p1, p4), df_mulf(p3, p2));
-    const dfl c11 = df_sub(df_mul(p0, p5), df_2prod(p2, p2));
-    const dfl c12 = df_sub(df_2prod(p1, p2), df_mulf(p0, p4));
-    const dfl c22 = df_sub(df_mul(p0, p3), df_2prod(p1, p1));
-    const dfl det = df_add(df_add(df_mul(p0, c00), df_mul(P1, c01)), df_mul(P2, c02));
+    // elimination of the scaled P: P = L diag(p0, d1, d2) L^T
+    const dfl p[6] = {p0, {p1, 0.0f}, {p2, 0.0f}, p3, {p4, 0.0f}, p5};
+    const dfl r0 = df_rcp(p0), l1 = df_mulf(r0, p1), l2 = df_mulf(r0, p2);
+    const dfl d1 = df_sub(p3, df_mulf(l1, p1)), e4 = df_sub(p[4], df_mulf(l1, p2));
+    const dfl r1 = df_rcp(d1), l3 = df_mul(e4, r1);
+    const dfl d2 = df_sub(df_sub(p5, df_mulf(l2, p2)), df_mul(l3, e4));
     dfl t[3] = {{x.x, 0.0f}, {x.y, 0.0f}, {x.z, 0.0f}};
-    if (det.hi != 0.0f && isfinite(det.hi)) {
-        const dfl f = df_mulf(df_rcp(det), P.lambda * sc);   // lambda sc / det
-        const dfl u0 = df_add(df_add(df_mulf(c00, acc[0]), df_mulf(c01, acc[1])), df_mulf(c02, acc[2]));
-        const dfl u1 = df_add(df_add(df_mulf(c01, acc[0]), df_mulf(c11, acc[1])), df_mulf(c12, acc[2]));
-        const dfl u2 = df_add(df_add(df_mulf(c02, acc[0]), df_mulf(c12, acc[1])), df_mulf(c22, acc[2]));
+    if (p0.hi != 0.0f && d1.hi != 0.0f && d2.hi != 0.0f && isfinite(p0.hi) && isfinite(d1.hi) && isfinite(d2.hi)) {
+        const dfl y1 = df_sub(dfl{acc[1], 0.0f}, df_mulf(l1, acc[0]));
+        const dfl y2 = df_sub(df_sub(dfl{acc[2], 0.0f}, df_mulf(l2, acc[0])), df_mul(l3, y1));
+        const dfl u2 = df_mul(y2, df_rcp(d2));
+        const dfl u1 = df_sub(df_mul(y1, r1), df_mul(l3, u2));
+        const dfl u0 = df_sub(df_sub(df_mulf(r0, acc[0]), df_mul(l1, u1)), df_mul(l2, u2));
+        const dfl f = df_2prod(P.lambda, sc);   // exact: sc is a power of two
         t[0] = df_sub(t[0], df_mul(u0, f));
         t[1] = df_sub(t[1], df_mul(u1, f));
         t[2] = df_sub(t[2], df_mul(u2, f));
@@ -1084,20 +1187,22 @@ __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, 
     float xo3[3] = {df_f(t[0]), df_f(t[1]), df_f(t[2])};
     if (P.use_box && (xo3[0] < P.lo[0] || xo3[0] > P.hi[0] || xo3[1] < P.lo[1] || xo3[1] > P.hi[1] ||
                       xo3[2] < P.lo[2] || xo3[2] > P.hi[2])) {
-        const double il = 1.0 / (double)P.lambda;
-        double T[6] = {acc[3] * il, acc[4] * il, acc[5] * il, acc[6] * il, acc[7] * il, acc[8] * il};
-        const double tr = T[0] + T[3] + T[5];
-        T[0] += 1e-12 * tr;
-        T[3] += 1e-12 * tr;
-        T[5] += 1e-12 * tr;
-        const double Q[3][3] = {{T[0], T[1], T[2]}, {T[1], T[3], T[4]}, {T[2], T[4], T[5]}};
-        const double td[3] = {(double)t[0].hi + (double)t[0].lo, (double)t[1].hi + (double)t[1].lo,
-                              (double)t[2].hi + (double)t[2].lo};
-        double xo[3];
-        box_prox3(Q, td, P.lo, P.hi, xo);
-        xo3[0] = (float)xo[0];
-        xo3[1] = (float)xo[1];
-        xo3[2] = (float)xo[2];
+        if (!box_step3(p, t, P.lo, P.hi, xo3)) {
+            const double il = 1.0 / (double)P.lambda;
+            double T[6] = {acc[3] * il, acc[4] * il, acc[5] * il, acc[6] * il, acc[7] * il, acc[8] * il};
+            const double tr = T[0] + T[3] + T[5];
+            T[0] += 1e-12 * tr;
+            T[3] += 1e-12 * tr;
+            T[5] += 1e-12 * tr;
+            const double Q[3][3] = {{T[0], T[1], T[2]}, {T[1], T[3], T[4]}, {T[2], T[4], T[5]}};
+            const double td[3] = {(double)t[0].hi + (double)t[0].lo, (double)t[1].hi + (double)t[1].lo,
+                                  (double)t[2].hi + (double)t[2].lo};
+            double xo[3];
+            box_prox3(Q, td, P.lo, P.hi, xo);
+            xo3[0] = (float)xo[0];
+            xo3[1] = (float)xo[1];
+            xo3[2] = (float)xo[2];
+        }
     }
     const float4 xn = make_float4(xo3[0], xo3[1], xo3[2], 0.f);
     D.x[k] = xn;
@@ -1607,8 +1712,9 @@ __device__ __forceinline__ void fpb_sum(const float* __restrict__ part, int G, s
 
 // The view groups' channels added in group order (as bp_finish does), then a7
 // for every pixel; PARTIAL: the sum goes to chan ([9][P]) instead.
+constexpr int kFinishThreads = 64;   // small blocks: a 64 x 64 image spreads over 64 SMs instead of 16
 template <bool PARTIAL>
-__global__ void k_fpb_finish(GeomC C, StepParams P, SolveD D, const float* __restrict__ part, int G, float* chan) {
+__global__ void __launch_bounds__(kFinishThreads) k_fpb_finish(GeomC C, StepParams P, SolveD D, const float* __restrict__ part, int G, float* chan) {
     const int P_ = C.grid.n * C.grid.n;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= P_) return;
@@ -1821,7 +1927,8 @@ cudaError_t launch_fpb(const GeomC& C, const FpTables& T, const RayRec* rec, con
     k_fpb_bp<PARTIAL><<<bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, smem, st>>>(C, T, rec, v0, v1, T.bp_part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_fpb_finish<PARTIAL><<<blocks(C.grid.n * C.grid.n, 256), 256, 0, st>>>(C, P, D, T.bp_part, T.bp_groups, chan);
+    k_fpb_finish<PARTIAL><<<blocks(C.grid.n * C.grid.n, kFinishThreads), kFinishThreads, 0, st>>>(C, P, D, T.bp_part,
+                                                                                            T.bp_groups, chan);
     return cudaGetLastError();
 }
 
