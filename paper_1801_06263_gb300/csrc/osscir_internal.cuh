@@ -317,24 +317,27 @@ struct GeomC {
     float margin_bins;       // candidate margin for the pixel-driven enumeration
 };
 
-// Candidate bin range of pixel (ix, iy) in a view: bins whose centre ray can
-// cross the pixel square (FP32 shadow of the four corners, with a margin).
+// Candidate bin range of pixel (ix, iy) in a view: bins whose centre ray can cross
+// the pixel square (a superset of its shadow, in FP32 with a margin; x_weight decides).
+// With num = q . e_u and den = sid - q . e at the pixel's centre, a corner at
+// (+-h/2, +-h/2) from it moves beta by scale (dx (c num - s den) + dy (c den + s num)) /
+// (den den'), den' the corner's own den, so half the shadow's width is at most
+// scale h/2 (|c num - s den| + |c den + s num|) / (den min den').  One point and two
+// divisions instead of the four corners': about 25 instructions instead of 55 for
+// each of the pixel-views that the pixel-driven kernels visit; the bound is wider
+// than the shadow by a factor h / den at most (0.1 % at 256 x 256).
 __device__ __forceinline__ void pixel_bin_range(const GeomC& C, const ViewF& V, int ix, int iy, int& blo,
                                                 int& bhi) {
-    const float X0 = grid_plane(C.grid, ix), X1 = grid_plane(C.grid, ix + 1);
-    const float Y0 = grid_plane(C.grid, iy), Y1 = grid_plane(C.grid, iy + 1);
-    float bmin = 3.0e38f, bmax = -3.0e38f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float X = (q & 1) ? X1 : X0, Y = (q & 2) ? Y1 : Y0;
-        const float num = -V.s * X + V.c * Y;
-        const float den = C.sid - (V.c * X + V.s * Y);
-        const float beta = C.scale * __fdividef(num, den) + C.mid;   // 2-ulp division; the margin covers it
-        bmin = fminf(bmin, beta);
-        bmax = fmaxf(bmax, beta);
-    }
-    blo = max(0, -sat_floor(-(bmin - C.margin_bins)));
-    bhi = min(C.n_bins - 1, sat_floor(bmax + C.margin_bins));
+    const float hh = 0.5f * C.grid.h;
+    const float X = grid_plane(C.grid, ix) + hh, Y = grid_plane(C.grid, iy) + hh;
+    const float num = fmaf(V.c, Y, -V.s * X), den = C.sid - fmaf(V.c, X, V.s * Y);
+    const float den_min = fmaxf(fmaf(-hh, fabsf(V.c) + fabsf(V.s), den), 1e-6f * den);
+    const float reach = fabsf(fmaf(V.c, num, -V.s * den)) + fabsf(fmaf(V.c, den, V.s * num));
+    // __fdividef is within 2 ulp; the margin covers it
+    const float beta = fmaf(C.scale, __fdividef(num, den), C.mid);
+    const float half = fmaf(C.scale * hh, __fdividef(reach, den * den_min), C.margin_bins);
+    blo = max(0, -sat_floor(half - beta));
+    bhi = min(C.n_bins - 1, sat_floor(beta + half));
 }
 
 }  // namespace osscir

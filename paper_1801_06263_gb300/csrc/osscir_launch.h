@@ -59,9 +59,8 @@ struct SolveD {
 constexpr int kModelStride = 11;
 
 constexpr int kFwdThreads = 128;
-constexpr int kBpTileX = 16, kBpTileY = 8;            // plain back-projection tile
 constexpr int kBpPixX = 2, kBpPixY = 32;              // MOCCA back-projection pixel tile (2 x 32: measured fastest)
-constexpr int kBpPix = kBpPixX * kBpPixY;
+constexpr int kBpPix = kBpPixX * kBpPixY;                // also the plain back-projection's pixels per block
 constexpr int kBpMaxThreads = 512;                    // kBpPix x up to 8 view groups
 // Blocked back-projection table: a block is a tile of kBTX x kBTY pixels (one
 // per thread) and one view group; its views go in chunks of at most kBTMaxChunk.
