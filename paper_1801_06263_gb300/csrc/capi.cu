@@ -54,8 +54,8 @@ void free_ctx(osscir_ctx* h) {
     void* ptrs[] = {h->rec,     h->r64,    h->views,     h->chord,    h->exc_off,    h->exc_ent,  h->s4,
                     h->N4,      h->mu,     h->mu_in,     h->g,        h->c,          h->y,        h->x,
                     h->xbar,    h->xo,     h->dtpl_part, h->dtpl_out, h->bad_counts, h->model,    h->fwd_row,
-                    h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_row,  h->bp_w,
-                    h->bp_slot, h->bp_roff,   h->bp_rays, h->bp_part};
+                    h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit, h->bp_w,
+                    h->bp_slot, h->bp_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete h;
@@ -263,7 +263,7 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
 
     const int L = h->L, P = h->P, nE = h->nE;
     h->n_part = dtpl_partials(g->n_bins, g->n_views);
-    CK(dalloc(&h->rec, 2 * (size_t)L));   // weight halves, then step halves
+    CK(dalloc(&h->rec, ray_recs(L)));   // weight halves, step halves, S22
     CK(dalloc(&h->r64, L));
     CK(dalloc(&h->views, g->n_views));
     CK(dalloc(&h->chord, L));
@@ -345,8 +345,8 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
 }
 
 void free_tables(osscir_ctx* h) {
-    void* ptrs[] = {h->fwd_row, h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_row,
-                    h->bp_w,    h->bp_slot, h->bp_roff,   h->bp_rays, h->bp_part};
+    void* ptrs[] = {h->fwd_row, h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit,
+                    h->bp_w,    h->bp_slot, h->bp_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     h->fwd_row = nullptr;
@@ -355,11 +355,9 @@ void free_tables(osscir_ctx* h) {
     h->fwd_w = nullptr;
     h->fwd_d = nullptr;
     h->bp_span = nullptr;
-    h->bp_row = nullptr;
+    h->bp_unit = nullptr;
     h->bp_w = nullptr;
     h->bp_slot = nullptr;
-    h->bp_roff = nullptr;
-    h->bp_rays = nullptr;
     h->bp_part = nullptr;
     h->bytes -= h->fp_bytes;
     h->fp_bytes = 0;
@@ -434,84 +432,48 @@ osscir_status build_tables(osscir_ctx* h) {
         CKT(e);
         if (bad_h) return fail(cudaErrorMemoryAllocation);
     }
-    // back-projection (blocked): per tile and view the union of candidate bins; the
-    // chunk size (views per staged chunk) so that two stage buffers fit in 48 KB;
-    // then per-pixel counts and per-warp rows of each (block, chunk), then the pairs
+    // back-projection (blocked): per tile and view the bins that can meet it; the chunk
+    // size (views per staged chunk) whose two stage buffers fit; the units of each
+    // (block, warp, chunk) and their prefix sum; then the entries
     const int n_t = bt_tiles(C.grid.n), per = (C.n_views + G - 1) / G;
     CKT(dalloc(&h->bp_span, (size_t)n_t * C.n_views));
-    CKT(launch_fpb_span(C, h->views, h->bp_span, st));
-    std::vector<uint32_t> span((size_t)n_t * C.n_views);
-    CKT(cudaMemcpyAsync(span.data(), h->bp_span, sizeof(uint32_t) * span.size(), cudaMemcpyDeviceToHost, st));
-    CKT(cudaStreamSynchronize(st));
-    int chunk = 0, slots = 0;
-    auto group_range = [&](int g, int& v0, int& v1) {
-        v0 = std::min(C.n_views, g * per);
-        v1 = std::min(C.n_views, v0 + per);
+    struct {
+        unsigned long long total;
+        int most[kBTSizes], wide;
+    } stat{};
+    int* stat_d = nullptr;
+    CKT(dalloc(&stat_d, sizeof stat / sizeof(int)));
+    unsigned long long* total_d = reinterpret_cast<unsigned long long*>(stat_d);
+    cudaError_t e = cudaMemsetAsync(stat_d, 0, sizeof stat, st);
+    auto read_stat = [&]() {
+        cudaError_t r = cudaMemcpyAsync(&stat, stat_d, sizeof stat, cudaMemcpyDeviceToHost, st);
+        return r != cudaSuccess ? r : cudaStreamSynchronize(st);
     };
-    for (int cand = kBTMaxChunk; cand >= 1 && !chunk; cand /= 2) {
-        int most = 0;
-        for (int t = 0; t < n_t; ++t)
-            for (int g = 0; g < G; ++g) {
-                int v0, v1;
-                group_range(g, v0, v1);
-                for (int u0 = v0; u0 < v1; u0 += cand) {
-                    int sum = 0;
-                    for (int u = u0; u < std::min(v1, u0 + cand); ++u)
-                        sum += (int)(span[(size_t)t * C.n_views + u] >> 16);
-                    most = std::max(most, sum);
-                }
-            }
-        const int padded = (most + 3) / 4 * 4;   // stage buffers of 44-byte slots stay 16-byte aligned
-        if (fpb_stage_bytes(padded) <= 48 * 1024) {
-            chunk = cand;
-            slots = padded;
-        }
-    }
-    if (chunk > 0) {
-        const int nch = (per + chunk - 1) / chunk;
-        const size_t n_e = (size_t)n_t * G * nch;
-        // each entry's staged rays, view after view, in slot order
-        std::vector<uint32_t> roff(n_e + 1, 0);
-        std::vector<int> rays;
-        for (int t = 0; t < n_t; ++t)
-            for (int g = 0; g < G; ++g) {
-                int v0, v1;
-                group_range(g, v0, v1);
-                for (int c = 0; c < nch; ++c) {
-                    roff[((size_t)t * G + g) * nch + c] = (uint32_t)rays.size();
-                    const int u0 = std::min(v1, v0 + c * chunk), u1 = std::min(v1, u0 + chunk);
-                    for (int u = u0; u < u1; ++u) {
-                        const uint32_t sp = span[(size_t)t * C.n_views + u];
-                        for (uint32_t i = 0; i < (sp >> 16); ++i) rays.push_back(u * C.n_bins + (int)(sp & 0xffffu) + (int)i);
-                    }
-                }
-            }
-        roff[n_e] = (uint32_t)rays.size();
-        CKT(dalloc(&h->bp_roff, n_e + 1));
-        CKT(dalloc(&h->bp_rays, rays.size()));
-        CKT(cudaMemcpyAsync(h->bp_roff, roff.data(), sizeof(uint32_t) * (n_e + 1), cudaMemcpyHostToDevice, st));
-        CKT(cudaMemcpyAsync(h->bp_rays, rays.data(), sizeof(int) * rays.size(), cudaMemcpyHostToDevice, st));
-        CKT(dalloc(&h->bp_row, n_e * (kBTThreads / 32) + 1));
-        CKT(launch_fpb_count(C, h->exc(), h->rec, h->views, G, chunk, nch, h->bp_row, st));
-        const size_t n_w = n_e * (kBTThreads / 32);
-        std::vector<uint32_t> brow(n_w + 1, 0);
-        CKT(cudaMemcpyAsync(brow.data(), h->bp_row, sizeof(uint32_t) * n_w, cudaMemcpyDeviceToHost, st));
-        CKT(cudaStreamSynchronize(st));
-        for (size_t i = 0; i < n_w; ++i) brow[i] = (brow[i] + 1) & ~1u;   // even: entries are read two at a time
-        if (!prefix_rows(brow, n_w)) return fail(cudaErrorMemoryAllocation);
-        CKT(cudaMemcpyAsync(h->bp_row, brow.data(), sizeof(uint32_t) * (n_w + 1), cudaMemcpyHostToDevice, st));
-        CKT(dalloc(&h->bp_w, (size_t)brow[n_w] * 32));
-        CKT(dalloc(&h->bp_slot, (size_t)brow[n_w] * 32));
-        CKT(dalloc(&h->bp_part, (size_t)G * 9 * h->P));
-        // rows a pixel does not fill: no slot (0xffff), weight 0
-        CKT(cudaMemsetAsync(h->bp_slot, 0xff, sizeof(uint16_t) * (size_t)brow[n_w] * 32, st));
-        CKT(cudaMemsetAsync(h->bp_w, 0, sizeof(float) * (size_t)brow[n_w] * 32, st));
-        CKT(launch_fpb_fill(C, h->exc(), h->rec, h->views, h->bp_span, G, chunk, nch, h->bp_row, h->bp_w,
-                            h->bp_slot, st));
+    if (e == cudaSuccess) e = launch_fpb_span(C, h->views, G, h->bp_span, stat_d + 2, st);
+    if (e == cudaSuccess) e = read_stat();
+    int chunk = 0;
+    for (int i = kBTSizes - 1; i >= 0 && !chunk && C.n_bins <= 65535; --i)   // bp_span holds a bin in 16 bits
+        if (stat.most[i] <= kBTSlots) chunk = bt_size(i);
+    if (e == cudaSuccess && chunk > 0) {
+        h->bp_groups = G;
         h->bp_chunk = chunk;
-        h->bp_nch = nch;
-        h->bp_slots = slots;
+        h->bp_nch = (per + chunk - 1) / chunk;
+        const size_t n_u = (size_t)n_t * G * kBTWarps * h->bp_nch;
+        e = dalloc(&h->bp_unit, n_u + 1);
+        if (e == cudaSuccess)
+            e = launch_fpb_count(C, h->exc(), h->rec, h->views, h->fp(), h->bp_unit, stat_d + 2 + kBTSizes, st);
+        if (e == cudaSuccess) e = launch_scan(h->bp_unit + 1, n_u, total_d, st);
+        if (e == cudaSuccess) e = read_stat();
+        if (e == cudaSuccess && stat.total > 0xffffffffull) e = cudaErrorMemoryAllocation;
+        h->bp_wide = stat.wide;
+        if (e == cudaSuccess) e = dalloc(&h->bp_part, (size_t)G * 9 * h->P);
+        if (e == cudaSuccess) e = dalloc(&h->bp_slot, ((size_t)stat.total + 1) * (stat.wide ? 64 : 32));
+        if (e == cudaSuccess) e = dalloc(&h->bp_w, ((size_t)stat.total + 1) * 64);   // one more unit: it is loaded ahead
+        if (e == cudaSuccess) e = launch_fpb_fill(C, h->exc(), h->rec, h->views, h->fp(), h->bp_w, h->bp_slot, st);
     }
+    cudaFree(stat_d);
+    h->bytes -= sizeof stat;
+    CKT(e);
     CKT(cudaStreamSynchronize(st));
 #undef CKT
     g_dalloc_bytes = &g_dalloc_bytes_sink;

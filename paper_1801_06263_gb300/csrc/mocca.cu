@@ -119,15 +119,22 @@ __device__ __forceinline__ void sexp3(float x, bool expm, float& e0, float& e1, 
 // that allocate no L1 line (measured about 2 % faster at 256x256 and 1 % at
 // 512x512; the forward table's entries loaded so were 10 % slower and keep
 // ordinary loads).
-__device__ __forceinline__ float2 ld_stream(const float2* p) {
-    float2 v;
-    asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+__device__ __forceinline__ float4 ld_stream(const float4* p) {
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
     return v;
 }
-__device__ __forceinline__ ushort2 ld_stream(const ushort2* p) {
-    unsigned u;
+__device__ __forceinline__ uint32_t ld_stream(const uint32_t* p) {
+    uint32_t u;
     asm("ld.global.nc.L1::no_allocate.b32 %0, [%1];" : "=r"(u) : "l"(p));
-    return make_ushort2((unsigned short)(u & 0xffffu), (unsigned short)(u >> 16));
+    return u;
+}
+__device__ __forceinline__ uint2 ld_stream(const uint2* p) {
+    uint2 u;
+    asm("ld.global.nc.L1::no_allocate.v2.b32 {%0, %1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(p));
+    return u;
 }
 
 // Half of a ray record (32 bytes, 32-byte aligned) in one 256-bit load.
@@ -665,7 +672,6 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
     constexpr int F4 = win_f4<W>();
     double dsum = 0.0;
     {
-        const float4 r1 = rec[l].r1;
         const float4 gg = D.g[l];
         const float g0 = gg.x, g1 = gg.y, g2 = gg.z;
         // a2/a3, one pass over energies: D_w, the alpha_w numerators and per window
@@ -812,10 +818,11 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
                 Sm[5] += fabsf(al[w][2]);
             }
         }
-        rec[l].r1 = make_float4(r1.x, r1.y, bb[0], bb[1]);
-        RayStep* st = ray_steps(rec, C.n_views * C.n_bins) + l;
-        st->s0 = make_float4(bb[2], Sm[0], Sm[1], Sm[2]);
-        st->s1 = make_float4(Sm[3], Sm[4], Sm[5], 0.f);
+        const RaySteps st = ray_steps(rec, C.n_views * C.n_bins);
+        st.s0[l] = make_float4(bb[0], bb[1], bb[2], Sm[0]);
+        st.s1[l] = make_float4(Sm[1], Sm[2], Sm[3], Sm[4]);
+        st.s22[l] = Sm[5];
+        rec[l].r1.z = Sm[5];
     }
     return dsum;
 }
@@ -872,9 +879,8 @@ __global__ void __launch_bounds__(kFwdThreads) k_mocca_ray_inner(GeomC C, RayRec
     for (int w = 0; w < 4; ++w)
 #pragma unroll
         for (int m = 0; m < 3; ++m) bb[m] = fmaf(al[w][m], yo[w], bb[m]);
-    const float4 r1 = rec[l].r1;
-    rec[l].r1 = make_float4(r1.x, r1.y, bb[0], bb[1]);
-    ray_steps(rec, C.n_views * C.n_bins)[l].s0.x = bb[2];
+    float4* s0 = ray_steps(rec, C.n_views * C.n_bins).s0 + l;
+    *s0 = make_float4(bb[0], bb[1], bb[2], s0->w);
 }
 
 // Box-constrained primal step: argmin over lo <= x <= hi of 1/2 (x - t)^T Q (x - t),
@@ -1051,19 +1057,38 @@ __device__ __forceinline__ void bp_finish(const GeomC& C, const StepParams& P, c
 __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, const SolveD& D, int k,
                                            const float acc[9]);
 
-// The nine channels of one footprint pair (weight w != 0): K^T y' (from b in
-// r1.zw and s0.x) and the step matrix (s0.yzw, s1.xyz).
-__device__ __forceinline__ void bp_accumulate(float acc[9], float w, const float4& r1, const float4& s0,
-                                              const float4& s1) {
-    acc[0] = fmaf(w, r1.z, acc[0]);
-    acc[1] = fmaf(w, r1.w, acc[1]);
-    acc[2] = fmaf(w, s0.x, acc[2]);
-    acc[3] = fmaf(w, s0.y, acc[3]);
-    acc[4] = fmaf(w, s0.z, acc[4]);
-    acc[5] = fmaf(w, s0.w, acc[5]);
-    acc[6] = fmaf(w, s1.x, acc[6]);
-    acc[7] = fmaf(w, s1.y, acc[7]);
-    acc[8] = fmaf(w, s1.z, acc[8]);
+// The nine channels of one footprint pair (weight w != 0): K^T y' (b in s0.xyz) and the
+// step matrix (s0.w, s1, s22).
+__device__ __forceinline__ void bp_accumulate(float* acc, float w, const float4& s0, const float4& s1, float s22) {
+    acc[0] = fmaf(w, s0.x, acc[0]);
+    acc[1] = fmaf(w, s0.y, acc[1]);
+    acc[2] = fmaf(w, s0.z, acc[2]);
+    acc[3] = fmaf(w, s0.w, acc[3]);
+    acc[4] = fmaf(w, s1.x, acc[4]);
+    acc[5] = fmaf(w, s1.y, acc[5]);
+    acc[6] = fmaf(w, s1.z, acc[6]);
+    acc[7] = fmaf(w, s1.w, acc[7]);
+    acc[8] = fmaf(w, s22, acc[8]);
+}
+
+// The same for any weight, nothing added where w is zero (also where a record is not
+// finite): predicated multiply-adds, since a branch here costs the loads around it
+// their overlap (the whole kernel 235 us at 256 x 256 against 148 us).
+__device__ __forceinline__ void bp_accumulate_if(float* acc, float w, const float4& s0, const float4& s1, float s22) {
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.neu.f32 p, %9, 0f00000000;\n\t"
+        "@p fma.rn.f32 %0, %9, %10, %0;\n\t"
+        "@p fma.rn.f32 %1, %9, %11, %1;\n\t"
+        "@p fma.rn.f32 %2, %9, %12, %2;\n\t"
+        "@p fma.rn.f32 %3, %9, %13, %3;\n\t"
+        "@p fma.rn.f32 %4, %9, %14, %4;\n\t"
+        "@p fma.rn.f32 %5, %9, %15, %5;\n\t"
+        "@p fma.rn.f32 %6, %9, %16, %6;\n\t"
+        "@p fma.rn.f32 %7, %9, %17, %7;\n\t"
+        "@p fma.rn.f32 %8, %9, %18, %8;\n\t}"
+        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]), "+f"(acc[4]), "+f"(acc[5]), "+f"(acc[6]), "+f"(acc[7]),
+          "+f"(acc[8])
+        : "f"(w), "f"(s0.x), "f"(s0.y), "f"(s0.z), "f"(s0.w), "f"(s1.x), "f"(s1.y), "f"(s1.z), "f"(s1.w), "f"(s22));
 }
 
 // Pixel-driven back-projection of pixel (ix, iy) over the views [v0, v1):
@@ -1072,7 +1097,7 @@ __device__ __forceinline__ void bp_accumulate(float acc[9], float w, const float
 // nonzero ones.  Every form of the back-projection adds in this order.
 __device__ __forceinline__ void bp_pixel_sum(const GeomC& C, const ExcTable& E, const RayRec* rec,
                                              const ViewF* views, int ix, int iy, int v0, int v1, float acc[9]) {
-    const RayStep* steps = ray_steps(rec, C.n_views * C.n_bins);
+    const RaySteps steps = ray_steps(rec, C.n_views * C.n_bins);
     for (int v = v0; v < v1; ++v) {
         int blo, bhi;
         pixel_bin_range(C, views[v], ix, iy, blo, bhi);
@@ -1086,12 +1111,10 @@ __device__ __forceinline__ void bp_pixel_sum(const GeomC& C, const ExcTable& E, 
             const float wa = x_weight(A.a, A.b.x, A.b.y, C.grid, E, l, ix, iy);
             const float wb = two ? x_weight(B.a, B.b.x, B.b.y, C.grid, E, l + 1, ix, iy) : 0.0f;
             if (wa != 0.0f) {
-                const RecHalf A2 = ldg_half(&steps[l].s0);
-                bp_accumulate(acc, wa, A.b, A2.a, A2.b);
+                bp_accumulate(acc, wa, __ldg(steps.s0 + l), __ldg(steps.s1 + l), A.b.z);
             }
             if (wb != 0.0f) {
-                const RecHalf B2 = ldg_half(&steps[l + 1].s0);
-                bp_accumulate(acc, wb, B.b, B2.a, B2.b);
+                bp_accumulate(acc, wb, __ldg(steps.s0 + l + 1), __ldg(steps.s1 + l + 1), B.b.z);
             }
         }
     }
@@ -1402,54 +1425,46 @@ __global__ void __launch_bounds__(kFwdThreads, 8) k_fp_proj(GeomC C, FpTables T,
     if (l >= 0) fp_proj_ray(T, D, l, (l / C.n_bins) * ((C.n_bins + 31) >> 5) + bx);
 }
 
-// The footprint pairs of pixel (ix, iy) in the views [v0, v1), in the order
-// bp_pixel_sum adds them (views ascending, candidate bins ascending, nonzero
-// weights only): visit(l, w).
-template <class Visit>
-__device__ __forceinline__ void pixel_pairs(const GeomC& C, const ExcTable& E, const RayRec* rec,
-                                            const ViewF* views, int ix, int iy, int v0, int v1, Visit&& visit) {
-    for (int v = v0; v < v1; ++v) {
-        int blo, bhi;
-        pixel_bin_range(C, views[v], ix, iy, blo, bhi);
-        for (int b = blo; b <= bhi; ++b) {
-            const int l = v * C.n_bins + b;
-            const float4 r0 = rec[l].r0, r1 = rec[l].r1;
-            const float w = x_weight(r0, r1.x, r1.y, C.grid, E, l, ix, iy);
-            if (w != 0.0f) visit(l, w);
-        }
-    }
+__device__ __forceinline__ void cp_async16(uint32_t smem, const void* gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem), "l"(gmem) : "memory");
 }
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+__device__ __forceinline__ void cp_async4(uint32_t smem, const void* gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem), "l"(gmem) : "memory");
 }
 
 // ------------------------------------------------------------------ blocked back-projection table
 //
-// Block b = t G + g: pixel tile t (kBTX x kBTY pixels, one per thread) and view
+// Block b = t G + g: pixel tile t (kBTX x kBTY pixels, two per thread) and view
 // group g of G (the split of k_mocca_bp).  The group's views go in chunks of
-// T.bp_chunk views; for chunk c the block stages, with asynchronous 16-byte
-// copies, the records of the rays that can meet the tile (per view u the bins
-// [tlo_u, tlo_u + span_u) of bp_span, view after view: stage slot
-// off_u + b - tlo_u), and each pixel runs through its pairs (slot, weight) of
-// the chunk, in the order of bp_pixel_sum.  A ray's record is read from L2 once
-// per tile and view and then from shared memory by every pixel that meets it.
+// T.bp_chunk views; for each chunk the block stages, with asynchronous copies, the
+// step halves of the rays that can meet the tile (per view u the bins
+// [tlo_u, tlo_u + span_u) of bp_span, view after view), and each thread runs through
+// its entries (slot, weights of its two pixels) of the chunk.  A ray's record is
+// read from L2 once per tile and view and then from shared memory by every thread
+// that meets it.
+//
+// Why two pixels, one above the other, per thread: the kernel is bound by the
+// shared-memory reads of the staged records (36 bytes an entry, nine wavefronts a
+// warp row whatever the lanes share) and by its table stream.  A ray that meets a
+// pixel mostly meets the one above it too, so a pair takes about 2.9 rows per view
+// where two single pixels take 4.1, and an entry's slot serves two weights: 27 M
+// shared-memory wavefronts became 16 M and, with the kernel's address arithmetic and
+// latencies (see the notes below), 143 -> 109 us at 256 x 256 (512 x 512 rays) and
+// 1018 -> 683 us at 512 x 512 (1024 x 1024), group sums and step included.
 
-// The pixel of thread `tid` in tile t: warp w takes a 4 x 8 patch of the 16 x 16
-// tile (four patches across, two down), lane l pixel (l mod 4, l / 4) of it.  A
-// compact patch needs few neighbouring bins in any view, so the lanes' reads of
-// the staged slots at one table row hit few banks (measured: 0.147 ms against
-// 0.160 ms with a warp on two rows of 16, 0.156 ms with 8 x 4 patches).
+// The upper left (smaller iy) pixel of thread `tid` in tile t; its other pixel is
+// (ix, iy + 1).  Warp w takes an 8 x 8 patch of the tile and each quarter of it 4 x 4
+// pixels: a compact quarter needs few neighbouring bins in any view, so its lanes'
+// 16-byte reads of the staged slots at one row hit few banks.
 __device__ __forceinline__ void bt_pixel(int n, int t, int tid, int& ix, int& iy) {
-    static_assert(kBTX == 16 && kBTY == 16, "the warp patches tile 16 x 16");
-    const int ntx = (n + kBTX - 1) / kBTX, w = tid >> 5, l = tid & 31;
-    ix = (t % ntx) * kBTX + (w & 3) * 4 + (l & 3);
-    iy = (t / ntx) * kBTY + (w >> 2) * 8 + (l >> 2);
+    static_assert(kBTX == 16 && kBTY == 16 && kBTWarps == 4, "the warp patches tile 16 x 16");
+    const int ntx = (n + kBTX - 1) / kBTX, w = tid >> 5, q = (tid >> 3) & 3, i = tid & 7;
+    ix = (t % ntx) * kBTX + (w & 1) * 8 + (q & 1) * 4 + (i & 3);
+    iy = (t / ntx) * kBTY + (w >> 1) * 8 + (q >> 1) * 4 + (i >> 2) * 2;
 }
 
-// The views [u0, u1) of chunk c of group g (views [V0, V1) of the whole range
-// split as group_views does, then in chunks of `chunk`).
+// The views [u0, u1) of chunk c of group g (views [0, n_views) split as group_views
+// does, then in chunks of `chunk`).
 __device__ __forceinline__ void chunk_views(int n_views, int g, int G, int chunk, int c, int& u0, int& u1) {
     int v0, v1;
     group_views(0, n_views, g, G, v0, v1);
@@ -1457,197 +1472,257 @@ __device__ __forceinline__ void chunk_views(int n_views, int g, int G, int chunk
     u1 = min(v1, u0 + chunk);
 }
 
-// Table pass 0: per tile and view the union of its pixels' candidate bins,
-// tlo | span << 16 (span 0: no pixel of the tile has a candidate there).
-__global__ void __launch_bounds__(kBTThreads) k_fpb_span(GeomC C, const ViewF* views, uint32_t* span) {
-    __shared__ int red_lo[kBTThreads / 32], red_hi[kBTThreads / 32];
-    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    int ix, iy;
-    bt_pixel(C.grid.n, t, tid, ix, iy);
-    const bool valid = ix < C.grid.n && iy < C.grid.n;
-    for (int v = 0; v < C.n_views; ++v) {
-        int blo = 0x7fffffff, bhi = -1;
-        if (valid) {
-            int lo, hi;
-            pixel_bin_range(C, views[v], ix, iy, lo, hi);
-            if (lo <= hi) {
-                blo = lo;
-                bhi = hi;
-            }
-        }
-        blo = __reduce_min_sync(0xffffffffu, blo);
-        bhi = __reduce_max_sync(0xffffffffu, bhi);
-        if (lane == 0) {
-            red_lo[wid] = blo;
-            red_hi[wid] = bhi;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            int lo = red_lo[0], hi = red_hi[0];
-            for (int w = 1; w < kBTThreads / 32; ++w) {
-                lo = min(lo, red_lo[w]);
-                hi = max(hi, red_hi[w]);
-            }
-            span[(size_t)t * C.n_views + v] = hi < lo ? 0u : (uint32_t)lo | ((uint32_t)(hi - lo + 1) << 16);
-        }
-        __syncthreads();
-    }
+// Table pass 0: per tile and view the bins that can meet the tile, tlo | span << 16.
+__global__ void __launch_bounds__(256) k_fpb_span(GeomC C, const ViewF* views, uint32_t* span) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, n = C.grid.n;
+    const int ntx = (n + kBTX - 1) / kBTX, n_t = ntx * ((n + kBTY - 1) / kBTY);
+    if (i >= n_t * C.n_views) return;
+    const int t = i / C.n_views, v = i % C.n_views;
+    const int ix = (t % ntx) * kBTX, iy = (t / ntx) * kBTY;
+    const float X0 = grid_plane(C.grid, ix), X1 = grid_plane(C.grid, min(n, ix + kBTX));
+    const float Y0 = grid_plane(C.grid, iy), Y1 = grid_plane(C.grid, min(n, iy + kBTY));
+    int lo, hi;
+    box_bin_range(C, views[v], 0.5f * (X0 + X1), 0.5f * (Y0 + Y1), 0.5f * (X1 - X0), 0.5f * (Y1 - Y0), lo, hi);
+    span[i] = hi < lo ? 0u : (uint32_t)lo | ((uint32_t)(hi - lo + 1) << 16);
 }
 
-// The stage slot offsets of chunk views [u0, u1) of tile t: off[i] for view u0 + i.
-__device__ __forceinline__ int chunk_offsets(const uint32_t* span, int t, int n_views, int u0, int u1,
-                                             int off[kBTMaxChunk], int tlo[kBTMaxChunk], int wid[kBTMaxChunk]) {
+// The largest stage of any (tile, group, chunk) for every chunk size.
+__global__ void __launch_bounds__(128) k_fpb_most(GeomC C, const uint32_t* __restrict__ span, int G, int* most) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x, n = C.grid.n;
+    const int n_t = ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / kBTY);
+    if (b >= n_t * G) return;
+    int v0, v1, sum[kBTSizes], top[kBTSizes];
+    group_views(0, C.n_views, b % G, G, v0, v1);
+#pragma unroll
+    for (int s = 0; s < kBTSizes; ++s) sum[s] = top[s] = 0;
+    for (int v = v0; v < v1; ++v) {
+        const int w = (int)(span[(size_t)(b / G) * C.n_views + v] >> 16);
+#pragma unroll
+        for (int s = 0; s < kBTSizes; ++s) {
+            if ((v - v0) % bt_size(s) == 0) sum[s] = 0;
+            sum[s] += w;
+            top[s] = max(top[s], sum[s]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < kBTSizes; ++s) atomicMax(most + s, top[s]);
+}
+
+// Thread entries of view u: the bins from the first to the last that meets either of
+// its two pixels.  visit(l, w0, w1) for each; returns their number and the first bin.
+template <class Visit>
+__device__ __forceinline__ int pair_entries(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF& V,
+                                            int u, int ix, int iy, int& first, Visit&& visit) {
+    const float hh = 0.5f * C.grid.h;
+    const bool two = iy + 1 < C.grid.n;
+    int blo, bhi, cnt = 0, gap = 0;
+    first = 0;
+    box_bin_range(C, V, grid_plane(C.grid, ix) + hh, two ? grid_plane(C.grid, iy + 1) : grid_plane(C.grid, iy) + hh,
+                  hh, two ? C.grid.h : hh, blo, bhi);
+    for (int b = blo; b <= bhi; ++b) {
+        const int l = u * C.n_bins + b;
+        const float4 r0 = rec[l].r0, r1 = rec[l].r1;
+        const float w0 = x_weight(r0, r1.x, r1.y, C.grid, E, l, ix, iy);
+        const float w1 = two ? x_weight(r0, r1.x, r1.y, C.grid, E, l, ix, iy + 1) : 0.0f;
+        if (w0 == 0.0f && w1 == 0.0f) {
+            ++gap;
+            continue;
+        }
+        if (cnt == 0) first = b;
+        else
+            for (; gap > 0; --gap) visit(cnt++, 0.0f, 0.0f);   // a ray through a corner between two that count
+        gap = 0;
+        visit(cnt++, w0, w1);
+    }
+    return cnt;
+}
+
+// The stage slots of chunk views [u0, u1) of tile t: off[i] the first slot of view
+// u0 + i, tlo[i] its first bin.
+__device__ __forceinline__ void chunk_offsets(const uint32_t* span, int t, int n_views, int u0, int u1,
+                                              int off[kBTMaxChunk], int tlo[kBTMaxChunk]) {
     int total = 0;
 #pragma unroll
     for (int i = 0; i < kBTMaxChunk; ++i) {
-        const int u = u0 + i;
-        const uint32_t sp = u < u1 ? __ldg(span + (size_t)t * n_views + u) : 0u;
+        const uint32_t sp = u0 + i < u1 ? __ldg(span + (size_t)t * n_views + u0 + i) : 0u;
         off[i] = total;
         tlo[i] = (int)(sp & 0xffffu);
-        wid[i] = (int)(sp >> 16);
-        total += wid[i];
+        total += (int)(sp >> 16);
     }
-    return total;
 }
 
-// The table rows of a warp are aligned per view: view u of a chunk takes K_u rows,
-// the largest number of pairs any of the warp's pixels has in u, so that at every
-// row the warp's lanes read stage slots of one view (neighbouring slots, few bank
-// conflicts); a pixel with fewer pairs in u leaves the rest of them empty (slot
-// kBTNoSlot).
-constexpr uint16_t kBTNoSlot = 0xffff;
-
-// Table pass 1: per (block, chunk) and warp the number of rows, the sum of K_u.
+// Table pass 1: the units of each warp and chunk (see FpTables).
 __global__ void __launch_bounds__(kBTThreads) k_fpb_count(GeomC C, ExcTable E, const RayRec* rec,
-                                                          const ViewF* views, int G, int chunk, int nch,
-                                                          uint32_t* warp_rows) {
-    const int b = blockIdx.x, t = b / G, g = b % G, tid = threadIdx.x;
+                                                          const ViewF* views, FpTables T, uint32_t* unit, int* wide) {
+    const int G = T.bp_groups, nch = T.bp_nch, b = blockIdx.x, t = b / G, g = b % G, tid = threadIdx.x;
     int ix, iy;
     bt_pixel(C.grid.n, t, tid, ix, iy);
     const bool valid = ix < C.grid.n && iy < C.grid.n;
+    bool far = false;
+    if (b == 0 && tid == 0) unit[0] = 0;
     for (int c = 0; c < nch; ++c) {
-        int u0, u1;
-        chunk_views(C.n_views, g, G, chunk, c, u0, u1);
+        int u0, u1, off[kBTMaxChunk], tlo[kBTMaxChunk];
+        chunk_views(C.n_views, g, G, T.bp_chunk, c, u0, u1);
+        chunk_offsets(T.bp_span, t, C.n_views, u0, u1, off, tlo);
         uint32_t rows = 0;
+        int slot = 0;
         for (int u = u0; u < u1; ++u) {
-            int n = 0;
-            if (valid) pixel_pairs(C, E, rec, views, ix, iy, u, u + 1, [&](int, float) { ++n; });
+            int n = 0, first = 0;
+            if (valid) n = pair_entries(C, E, rec, views[u], u, ix, iy, first, [](int, float, float) {});
+            if (n > 0) {
+                const int s = off[u - u0] + first - tlo[u - u0];
+                far = far || s - slot < -128 || s - slot > 127;
+                slot = s + n - 1;
+            }
             rows += (uint32_t)__reduce_max_sync(0xffffffffu, n);
         }
-        const size_t e = (size_t)b * nch + c;
-        if ((tid & 31) == 0) warp_rows[e * (kBTThreads / 32) + (tid >> 5)] = rows;
+        if ((tid & 31) == 0) unit[1 + ((size_t)b * kBTWarps + (tid >> 5)) * nch + c] = (rows + 3) / 4;
     }
+    if (far) *wide = 1;
 }
 
-// Table pass 2: the pairs (stage slot, weight) at their rows: view u of the chunk
-// from the warp's row offset of u, pair j of a lane at row bp_row[(e, warp)] + j
-// (two rows side by side per lane).  The slots start as kBTNoSlot (memset).
+// Table pass 2: every row of every unit.
 __global__ void __launch_bounds__(kBTThreads) k_fpb_fill(GeomC C, ExcTable E, const RayRec* rec,
-                                                         const ViewF* views, const uint32_t* __restrict__ span,
-                                                         int G, int chunk, int nch,
-                                                         const uint32_t* __restrict__ bp_row, float* bp_w,
-                                                         uint16_t* bp_slot) {
-    const int b = blockIdx.x, t = b / G, g = b % G, tid = threadIdx.x, lane = tid & 31;
+                                                         const ViewF* views, FpTables T, float4* bp_w,
+                                                         uint32_t* bp_slot) {
+    const int G = T.bp_groups, nch = T.bp_nch, b = blockIdx.x, t = b / G, g = b % G, tid = threadIdx.x, lane = tid & 31;
     int ix, iy;
     bt_pixel(C.grid.n, t, tid, ix, iy);
     const bool valid = ix < C.grid.n && iy < C.grid.n;
+    const size_t ui = ((size_t)b * kBTWarps + (tid >> 5)) * nch;
     for (int c = 0; c < nch; ++c) {
-        int u0, u1;
-        chunk_views(C.n_views, g, G, chunk, c, u0, u1);
-        int off[kBTMaxChunk], tlo[kBTMaxChunk], wid[kBTMaxChunk];
-        chunk_offsets(span, t, C.n_views, u0, u1, off, tlo, wid);
-        const size_t e = (size_t)b * nch + c;
-        const size_t row = bp_row[e * (kBTThreads / 32) + (tid >> 5)];
-        int j0 = 0;   // the warp's first row of view u
+        int u0, u1, off[kBTMaxChunk], tlo[kBTMaxChunk];
+        chunk_views(C.n_views, g, G, T.bp_chunk, c, u0, u1);
+        chunk_offsets(T.bp_span, t, C.n_views, u0, u1, off, tlo);
+        const size_t q0 = T.bp_unit[ui + c], q1 = T.bp_unit[ui + c + 1];
+        int r = 0, slot = 0, prev = 0;   // the next row, its slot, the slot of the row before
+        auto put = [&](int s, float w0, float w1) {
+            const size_t q = q0 + (r >> 2);
+            reinterpret_cast<float2*>(bp_w + 64 * q + 32 * ((r >> 1) & 1) + lane)[r & 1] = make_float2(w0, w1);
+            if (T.bp_wide)
+                reinterpret_cast<uint16_t*>(bp_slot + 64 * q + 2 * lane)[r & 3] = (uint16_t)s;
+            else
+                reinterpret_cast<int8_t*>(bp_slot + 32 * q + lane)[r & 3] = (int8_t)(s - prev);
+            prev = s;
+            ++r;
+        };
         for (int u = u0; u < u1; ++u) {
-            int n = 0;
-            if (valid) pixel_pairs(C, E, rec, views, ix, iy, u, u + 1, [&](int, float) { ++n; });
+            int n = 0, first = 0;
+            if (valid) n = pair_entries(C, E, rec, views[u], u, ix, iy, first, [](int, float, float) {});
             const int K = __reduce_max_sync(0xffffffffu, n);
-            int j = j0;
-            if (valid)
-                pixel_pairs(C, E, rec, views, ix, iy, u, u + 1, [&](int l, float w) {
-                    const int i = u - u0;
-                    const int slot = off[i] + (l - u * C.n_bins) - tlo[i];
-                    const size_t at = (row + (j & ~1)) * 32 + 2 * lane + (j & 1);   // rows j, j + 1 side by side
-                    bp_w[at] = w;
-                    bp_slot[at] = (uint16_t)slot;
-                    ++j;
-                });
-            j0 += K;
+            if (n > 0) {
+                const int s0 = off[u - u0] + first - tlo[u - u0];
+                pair_entries(C, E, rec, views[u], u, ix, iy, first, [&](int j, float w0, float w1) { put(s0 + j, w0, w1); });
+                slot = s0 + n - 1;
+            }
+            for (int j = n; j < K; ++j) put(slot, 0.0f, 0.0f);
         }
+        while (r < 4 * (int)(q1 - q0)) put(slot, 0.0f, 0.0f);
     }
 }
 
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
+// A stage buffer of kBTSlots slots: s0 (b, S00) at its start, s1 (S01, S02, S11, S12) at
+// kBTStageS1 and s22 at kBTStageS22, addressed with 32-bit shared addresses (through
+// generic pointers the reads of a row cost twice the instructions).
+constexpr uint32_t kBTStageS1 = 16 * kBTSlots, kBTStageS22 = 32 * kBTSlots, kBTStage = 36 * kBTSlots;
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
 }
+__device__ __forceinline__ float lds1(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts1(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 
-// One stage buffer of S slots: the step halves (b2 and S in s0.x..s1.z), b0 and
-// b1 (the .zw of the weight half), and the ray index of each slot.
-struct StageBuf {
-    float4* s0;
-    float4* s1;
-    float2* b01;
-    int* ray;
-    __device__ StageBuf(float4* base, int S)
-        : s0(base), s1(base + S), b01(reinterpret_cast<float2*>(base + 2 * S)),
-          ray(reinterpret_cast<int*>(reinterpret_cast<float2*>(base + 2 * S) + S)) {}
-};
-// float4 units per stage buffer of S slots (S a multiple of 4: 44 S bytes).
-__host__ __device__ __forceinline__ int stage_f4(int S) { return (44 * S) / 16; }
-
-// Stage entry e's rays (bp_rays[bp_roff[e] ..]) into the buffer, asynchronously.
-__device__ __forceinline__ void stage_entry(const FpTables& T, const RayRec* rec, const RayStep* steps, size_t e,
-                                            StageBuf B) {
-    const uint32_t r0 = __ldg(T.bp_roff + e), nr = __ldg(T.bp_roff + e + 1) - r0;
-    for (uint32_t r = threadIdx.x; r < nr; r += kBTThreads) {
-        const int l = __ldg(T.bp_rays + r0 + r);
-        cp_async16(B.s0 + r, &steps[l].s0);
-        cp_async16(B.s1 + r, &steps[l].s1);
-        cp_async8(B.b01 + r, &rec[l].r1.z);
-        B.ray[r] = l;
+// Stage the rays of the views [u0, u1) that can meet a tile into the buffer at `buf`,
+// asynchronously: warp w copies views u0 + w, u0 + w + kBTWarps, ..., lane i bin i of
+// the view's run.  sp: lane i's bp_span of view u0 + i (0 beyond u1).  PARTIAL: the rays
+// of views outside [V0, V1) are staged as zeros, so they add nothing.
+template <bool PARTIAL>
+__device__ __forceinline__ void stage_views(const GeomC& C, const RaySteps& steps, uint32_t sp, int u0, int u1, int V0,
+                                            int V1, uint32_t buf) {
+    const int lane = threadIdx.x & 31;
+    int off = (int)(sp >> 16);
+#pragma unroll
+    for (int o = 1; o < kBTMaxChunk; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, off, o);
+        if (lane >= o) off += v;
+    }
+    off -= (int)(sp >> 16);
+    for (int i = threadIdx.x >> 5; i < u1 - u0; i += kBTWarps) {
+        const uint32_t si = __shfl_sync(0xffffffffu, sp, i);
+        const int oi = __shfl_sync(0xffffffffu, off, i), n = (int)(si >> 16);
+        const size_t l0 = (size_t)(u0 + i) * C.n_bins + (si & 0xffffu);
+        const bool out = PARTIAL && (u0 + i < V0 || u0 + i >= V1);
+        for (int p = lane; p < n; p += 32) {
+            const uint32_t a = buf + 16u * (oi + p), z = buf + kBTStageS22 + 4u * (oi + p);
+            const size_t l = l0 + p;
+            if (out) {
+                for (int j = 0; j < 4; ++j) {
+                    sts1(a + 4 * j, 0.f);
+                    sts1(a + kBTStageS1 + 4 * j, 0.f);
+                }
+                sts1(z, 0.f);
+            } else {
+                cp_async16(a, steps.s0 + l);
+                cp_async16(a + kBTStageS1, steps.s1 + l);
+                cp_async4(z, steps.s22 + l);
+            }
+        }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// The nine channels of one pair from a stage slot.
-__device__ __forceinline__ void bp_accumulate_slot(float acc[9], float w, const StageBuf& B, int s) {
-    const float2 b = B.b01[s];
-    const float4 s0 = B.s0[s], s1 = B.s1[s];
-    acc[0] = fmaf(w, b.x, acc[0]);
-    acc[1] = fmaf(w, b.y, acc[1]);
-    acc[2] = fmaf(w, s0.x, acc[2]);
-    acc[3] = fmaf(w, s0.y, acc[3]);
-    acc[4] = fmaf(w, s0.z, acc[4]);
-    acc[5] = fmaf(w, s0.w, acc[5]);
-    acc[6] = fmaf(w, s1.x, acc[6]);
-    acc[7] = fmaf(w, s1.y, acc[7]);
-    acc[8] = fmaf(w, s1.z, acc[8]);
+// Bytes (a multiple of 16, from a 16-byte boundary) on their way from HBM to L2.
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// a6 from the blocked table for block b = t G + g: each pixel's nine channels
-// over its group's views, written to part ([G][9][P]); the group sums and the
-// step follow in a second pass.  The chunks go through two stage buffers (smem):
-// chunk c + 1 is copied while chunk c is summed.  PARTIAL: only the rays of the
-// views [V0, V1) (one GPU's share of a split solve).  Every thread of the block
-// must call this (it contains block barriers).
-template <bool PARTIAL>
-__device__ __forceinline__ void fpb_block(const GeomC& C, const FpTables& T, const RayRec* rec, int V0, int V1,
-                                          float* part, int b, float4* smem) {
+// One unit of a lane: four rows' weights of its two pixels and their stage slots.
+template <bool WIDE>
+struct Unit {
+    float4 a, b;
+    uint32_t s[WIDE ? 2 : 1];
+};
+template <bool WIDE>
+__device__ __forceinline__ Unit<WIDE> ld_unit(const float4* w, const uint32_t* s) {
+    Unit<WIDE> r;
+    r.a = ld_stream(w);
+    r.b = ld_stream(w + 32);
+    if (WIDE) {
+        const uint2 v = ld_stream(reinterpret_cast<const uint2*>(s));
+        r.s[0] = v.x;
+        r.s[WIDE ? 1 : 0] = v.y;
+    } else {
+        r.s[0] = ld_stream(s);
+    }
+    return r;
+}
+
+// a6 from the blocked table for block b = t G + g: each thread's two pixels' nine
+// channels over its group's views, written to part ([G][9][P]); the group sums and
+// the step follow in a second pass.  The chunks go through two stage buffers (smem):
+// chunk c + 1 is copied while chunk c is summed, and the next unit's entries are
+// loaded while the current one's are added (one unit past the table's end is
+// allocated for that).  A pixel's additions are bp_pixel_sum's, in its order (views
+// ascending, bins ascending, nonzero weights only).  PARTIAL: only the rays of the
+// views [V0, V1) (one GPU's share of a split solve).  Every thread of the block must
+// call this (it contains block barriers).
+template <bool PARTIAL, bool WIDE>
+__device__ __forceinline__ void fpb_sum_block(const GeomC& C, const FpTables& T, const RayRec* rec, int V0, int V1,
+                                              float* part, int b, uint32_t smem) {
     const int G = T.bp_groups, t = b / G, g = b % G, tid = threadIdx.x, lane = tid & 31;
-    const int S = T.bp_slots, nch = T.bp_nch, nb = C.n_bins;
-    int ix, iy;
-    bt_pixel(C.grid.n, t, tid, ix, iy);
-    const bool valid = ix < C.grid.n && iy < C.grid.n;
-    const RayStep* steps = ray_steps(rec, C.n_views * nb);
-    const int l_lo = V0 * nb, l_hi = V1 * nb;
-    float acc[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const size_t e0 = (size_t)b * nch;
+    const int nch = T.bp_nch;
+    const RaySteps steps = ray_steps(rec, C.n_views * C.n_bins);
+    float acc[18];
+#pragma unroll
+    for (int i = 0; i < 18; ++i) acc[i] = 0.f;
     // PARTIAL: only the chunks whose views meet [V0, V1), a contiguous run of the
     // group's chunks (the same for every thread of the block), so a rank streams
-    // the table of its own views only; the per-slot test below keeps the rays of
-    // a chunk that straddles V0 or V1 apart
+    // the table of its own views only
     int c_lo = 0, c_hi = nch;
     if (PARTIAL) {
         c_lo = nch;
@@ -1661,63 +1736,124 @@ __device__ __forceinline__ void fpb_block(const GeomC& C, const FpTables& T, con
             }
         }
     }
-    const StageBuf B0(smem, S), B1(smem + stage_f4(S), S);
-    if (c_lo < c_hi) stage_entry(T, rec, steps, e0 + c_lo, (c_lo & 1) ? B1 : B0);
-    for (int c = c_lo; c < c_hi; ++c) {
-        const StageBuf& B = (c & 1) ? B1 : B0;
-        if (c + 1 < c_hi) {   // the next chunk into the other buffer (free since the barrier ending chunk c - 1)
-            stage_entry(T, rec, steps, e0 + c + 1, (c & 1) ? B0 : B1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncthreads();   // chunk c staged by every thread
-        const size_t e = e0 + c;
-        const uint32_t* rp = T.bp_row + e * (kBTThreads / 32) + (tid >> 5);
-        const size_t row = __ldg(rp);                  // even
-        const int n = (int)(__ldg(rp + 1) - row);      // the warp's rows (even): the same for every lane
-        const float2* wp = reinterpret_cast<const float2*>(T.bp_w + row * 32) + lane;
-        const ushort2* sp = reinterpret_cast<const ushort2*>(T.bp_slot + row * 32) + lane;
-        auto take = [&](float w, unsigned s) {
-            if (s != kBTNoSlot && (!PARTIAL || (B.ray[s] >= l_lo && B.ray[s] < l_hi))) bp_accumulate_slot(acc, w, B, s);
-        };
-        int j = 0;
-        for (; j + 7 < n; j += 8) {   // eight table entries (four loads of two) in flight
-            float2 w[4];
-            ushort2 sl[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                w[q] = ld_stream(wp + 32 * q);
-                sl[q] = ld_stream(sp + 32 * q);
+    auto span_of = [&](int c) {   // lane i: the span of the chunk's view i
+        int u0, u1;
+        chunk_views(C.n_views, g, G, T.bp_chunk, c, u0, u1);
+        return c < c_hi && u0 + lane < u1 ? __ldg(T.bp_span + (size_t)t * C.n_views + u0 + lane) : 0u;
+    };
+    auto stage = [&](int c, uint32_t sp) {
+        int u0, u1;
+        chunk_views(C.n_views, g, G, T.bp_chunk, c, u0, u1);
+        stage_views<PARTIAL>(C, steps, sp, u0, u1, V0, V1, smem + (c & 1) * kBTStage);
+    };
+    if (c_lo < c_hi) {
+        const uint32_t* up = T.bp_unit + ((size_t)b * kBTWarps + (tid >> 5)) * nch;
+        uint32_t sp = span_of(c_lo);
+        // the first unit of chunk c, of c + 1 and of c + 2: the same for every lane
+        uint32_t q = __ldg(up + c_lo), q1 = __ldg(up + c_lo + 1), q2 = c_lo + 1 < c_hi ? __ldg(up + c_lo + 2) : q1;
+        stage(c_lo, sp);
+        sp = span_of(c_lo + 1);
+        const float4* wp = T.bp_w + (size_t)64 * q + lane;
+        const uint32_t* dp = T.bp_slot + (WIDE ? (size_t)64 * q + 2 * lane : (size_t)32 * q + lane);
+        Unit<WIDE> next = ld_unit<WIDE>(wp, dp);
+        for (int c = c_lo; c < c_hi; ++c) {
+            if (c + 1 < c_hi) {   // the next chunk into the other buffer (free since the barrier ending chunk c - 1)
+                stage(c + 1, sp);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                take(w[q].x, sl[q].x);
-                take(w[q].y, sl[q].y);
+            __syncthreads();   // chunk c staged by every thread
+            sp = span_of(c + 2);
+            const uint32_t q3 = c + 2 < c_hi ? __ldg(up + c + 3) : q2;
+            if (lane == 0 && q2 > q1) {   // the next chunk's units on their way to L2
+                l2_prefetch(T.bp_w + (size_t)64 * q1, 1024u * (q2 - q1));
+                l2_prefetch(T.bp_slot + (size_t)(WIDE ? 64 : 32) * q1, (WIDE ? 256u : 128u) * (q2 - q1));
             }
-            wp += 128;
-            sp += 128;
+            // the addresses of the row's slot: its s0 (s1 at a constant distance) and its s22
+            uint32_t at = smem + (c & 1) * kBTStage, az = at + kBTStageS22;
+            const uint32_t at0 = at, az0 = az;
+            auto row = [&](float w0, float w1) {
+                const float4 s0 = lds4(at), s1 = lds4(at + kBTStageS1);
+                const float z = lds1(az);
+                bp_accumulate_if(acc, w0, s0, s1, z);
+                bp_accumulate_if(acc + 9, w1, s0, s1, z);
+            };
+            auto move = [&](const Unit<WIDE>& e, int r) {
+                if (WIDE) {
+                    const uint32_t s = (e.s[WIDE ? r >> 1 : 0] >> (16 * (r & 1))) & 0xffffu;
+                    at = at0 + 16 * s;
+                    az = az0 + 4 * s;
+                } else {
+                    const int d = (int8_t)(e.s[0] >> (8 * r));
+                    at += 16 * d;
+                    az += 4 * d;
+                }
+            };
+            auto unit = [&](const Unit<WIDE>& e) {
+                move(e, 0);
+                row(e.a.x, e.a.y);
+                move(e, 1);
+                row(e.a.z, e.a.w);
+                move(e, 2);
+                row(e.b.x, e.b.y);
+                move(e, 3);
+                row(e.b.z, e.b.w);
+            };
+            int k = (int)(q1 - q);
+#pragma unroll 1
+            for (; k > 1; k -= 2) {
+                const Unit<WIDE> second = ld_unit<WIDE>(wp + 64, dp + (WIDE ? 64 : 32));
+                unit(next);
+                wp += 128;
+                dp += WIDE ? 128 : 64;
+                next = ld_unit<WIDE>(wp, dp);
+                unit(second);
+            }
+            if (k > 0) {
+                const Unit<WIDE> e = next;
+                wp += 64;
+                dp += WIDE ? 64 : 32;
+                next = ld_unit<WIDE>(wp, dp);
+                unit(e);
+            }
+            q = q1;
+            q1 = q2;
+            q2 = q3;
+            __syncthreads();   // this buffer is read by everyone before chunk c + 2 overwrites it
         }
-        for (; j < n; j += 2, wp += 32, sp += 32) {
-            const float2 w = ld_stream(wp);
-            const ushort2 sl = ld_stream(sp);
-            take(w.x, sl.x);
-            take(w.y, sl.y);
-        }
-        __syncthreads();   // this buffer is read by everyone before chunk c + 2 overwrites it
     }
-    if (valid) {
+    int ix, iy;
+    bt_pixel(C.grid.n, t, tid, ix, iy);
+    if (ix < C.grid.n && iy < C.grid.n) {
         const size_t P_ = (size_t)C.grid.n * C.grid.n, k = (size_t)iy * C.grid.n + ix;
+        const bool two = iy + 1 < C.grid.n;
 #pragma unroll
-        for (int ch = 0; ch < 9; ++ch) part[((size_t)g * 9 + ch) * P_ + k] = acc[ch];
+        for (int ch = 0; ch < 9; ++ch) {
+            float* p = part + ((size_t)g * 9 + ch) * P_ + k;
+            p[0] = acc[ch];
+            if (two) p[C.grid.n] = acc[9 + ch];
+        }
     }
 }
 
 template <bool PARTIAL>
-__global__ void __launch_bounds__(kBTThreads) k_fpb_bp(GeomC C, FpTables T, const RayRec* rec, int V0, int V1,
+__device__ __forceinline__ void fpb_block(const GeomC& C, const FpTables& T, const RayRec* rec, int V0, int V1,
+                                          float* part, int b) {
+    __shared__ float4 stage[2 * kBTStage / 16];
+    const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(stage));
+    if (T.bp_wide) fpb_sum_block<PARTIAL, true>(C, T, rec, V0, V1, part, b, sa);
+    else fpb_sum_block<PARTIAL, false>(C, T, rec, V0, V1, part, b, sa);
+}
+
+// Seven resident blocks (72 registers, a handful of spilled words): 109 us at 256 x 256
+// with the step and 683 us at 512 x 512, against 115 and 707 with six; eight (64
+// registers) were slower.
+constexpr int kBTResident = 7;
+template <bool PARTIAL>
+__global__ void __launch_bounds__(kBTThreads, kBTResident) k_fpb_bp(GeomC C, FpTables T, const RayRec* rec, int V0, int V1,
                                                        float* part) {
-    extern __shared__ float4 bt_smem[];   // two stage buffers
-    fpb_block<PARTIAL>(C, T, rec, V0, V1, part, blockIdx.x, bt_smem);
+    fpb_block<PARTIAL>(C, T, rec, V0, V1, part, blockIdx.x);
 }
 
 // The view groups of pixel k added in group order (as bp_finish does).
@@ -1745,6 +1881,48 @@ __global__ void __launch_bounds__(kFinishThreads) k_fpb_finish(GeomC C, StepPara
     } else {
         pixel_step(C, P, D, k, acc);
     }
+}
+
+// In-place inclusive prefix sum by one block: each thread takes kScanEach
+// consecutive values of a tile, the tiles follow one another.
+constexpr int kScanThreads = 1024, kScanEach = 16;
+__global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* v, size_t n, unsigned long long* total) {
+    __shared__ unsigned long long warp_sum[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned long long carry = 0;
+    for (size_t base = 0; base < n; base += (size_t)kScanThreads * kScanEach) {
+        const size_t i0 = base + (size_t)threadIdx.x * kScanEach;
+        uint32_t x[kScanEach];
+        unsigned long long own = 0;
+#pragma unroll
+        for (int j = 0; j < kScanEach; ++j) {
+            x[j] = i0 + j < n ? v[i0 + j] : 0u;
+            own += x[j];
+        }
+        unsigned long long inc = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) warp_sum[wid] = inc;
+        __syncthreads();
+        unsigned long long before = carry, all = 0;
+        for (int w = 0; w < kScanThreads / 32; ++w) {
+            const unsigned long long u = warp_sum[w];
+            before += w < wid ? u : 0ull;
+            all += u;
+        }
+        carry += all;
+        unsigned long long run = before + inc - own;
+#pragma unroll
+        for (int j = 0; j < kScanEach; ++j) {
+            run += x[j];
+            if (i0 + j < n) v[i0 + j] = (uint32_t)run;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *total = carry;
 }
 
 constexpr int kReduceThreads = 1024;
@@ -1798,14 +1976,13 @@ __global__ void __launch_bounds__(kBatchProjMaxThreads) k_batch_proj(const Solve
 }
 
 // Batched back-projection from the solves' blocked tables: item (solve, block b)
-// runs fpb_block; the dynamic shared memory holds the largest solve's stages.
-__global__ void __launch_bounds__(kBTThreads) k_batch_fpb_bp(const SolveDesc* __restrict__ sd,
+// runs fpb_block.
+__global__ void __launch_bounds__(kBTThreads, kBTResident) k_batch_fpb_bp(const SolveDesc* __restrict__ sd,
                                                              const int2* __restrict__ items, int n_items) {
-    extern __shared__ float4 bt_smem[];
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
         const int2 w = __ldg(items + it);
         const SolveDesc& d = sd[w.x];
-        fpb_block<false>(d.C, d.T, d.rec, 0, d.C.n_views, d.T.bp_part, w.y, bt_smem);
+        fpb_block<false>(d.C, d.T, d.rec, 0, d.C.n_views, d.T.bp_part, w.y);
     }
 }
 
@@ -1943,8 +2120,7 @@ cudaError_t launch_mocca_ray_inner(const GeomC& C, RayRec* rec, const SolveD& D,
 template <bool PARTIAL>
 cudaError_t launch_fpb(const GeomC& C, const FpTables& T, const RayRec* rec, const StepParams& P, const SolveD& D,
                        int v0, int v1, float* chan, cudaStream_t st) {
-    const size_t smem = sizeof(float4) * 2 * (size_t)stage_f4(T.bp_slots);
-    k_fpb_bp<PARTIAL><<<bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, smem, st>>>(C, T, rec, v0, v1, T.bp_part);
+    k_fpb_bp<PARTIAL><<<bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, 0, st>>>(C, T, rec, v0, v1, T.bp_part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_fpb_finish<PARTIAL><<<blocks(C.grid.n * C.grid.n, kFinishThreads), kFinishThreads, 0, st>>>(C, P, D, T.bp_part,
@@ -1991,26 +2167,30 @@ cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* 
                                                                          bad);
     return cudaGetLastError();
 }
-cudaError_t launch_fpb_span(const GeomC& C, const ViewF* views, uint32_t* span, cudaStream_t st) {
-    k_fpb_span<<<bt_tiles(C.grid.n), kBTThreads, 0, st>>>(C, views, span);
+cudaError_t launch_fpb_span(const GeomC& C, const ViewF* views, int G, uint32_t* span, int* most, cudaStream_t st) {
+    k_fpb_span<<<blocks(bt_tiles(C.grid.n) * C.n_views, 256), 256, 0, st>>>(C, views, span);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_fpb_most<<<blocks(bt_tiles(C.grid.n) * G, 128), 128, 0, st>>>(C, span, G, most);
     return cudaGetLastError();
 }
 
-cudaError_t launch_fpb_count(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views, int G,
-                             int chunk, int nch, uint32_t* warp_rows, cudaStream_t st) {
-    k_fpb_count<<<bt_tiles(C.grid.n) * G, kBTThreads, 0, st>>>(C, E, rec, views, G, chunk, nch, warp_rows);
+cudaError_t launch_fpb_count(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
+                             const FpTables& T, uint32_t* unit, int* wide, cudaStream_t st) {
+    k_fpb_count<<<bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, 0, st>>>(C, E, rec, views, T, unit, wide);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fpb_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
-                            const uint32_t* span, int G, int chunk, int nch, const uint32_t* bp_row, float* bp_w,
-                            uint16_t* bp_slot, cudaStream_t st) {
-    k_fpb_fill<<<bt_tiles(C.grid.n) * G, kBTThreads, 0, st>>>(C, E, rec, views, span, G, chunk, nch, bp_row, bp_w,
-                                                               bp_slot);
+                            const FpTables& T, float4* bp_w, uint32_t* bp_slot, cudaStream_t st) {
+    k_fpb_fill<<<bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, 0, st>>>(C, E, rec, views, T, bp_w, bp_slot);
     return cudaGetLastError();
 }
 
-int fpb_stage_bytes(int slots) { return 2 * 16 * stage_f4(slots); }
+cudaError_t launch_scan(uint32_t* v, size_t n, unsigned long long* total, cudaStream_t st) {
+    k_scan<<<1, kScanThreads, 0, st>>>(v, n, total);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_mocca_apply(const GeomC& C, const StepParams& P, const SolveD& D, const float* chan,
                                cudaStream_t st) {
@@ -2050,9 +2230,9 @@ cudaError_t launch_batch_dtpl(const SolveDesc* sd, int n_solves, cudaStream_t st
 }
 
 cudaError_t launch_batch_fpb(const SolveDesc* sd, const int2* items, int n_items, const int2* fin_items,
-                             int n_fin, int grid, size_t smem, cudaStream_t st) {
+                             int n_fin, int grid, cudaStream_t st) {
     if (n_items > 0) {
-        k_batch_fpb_bp<<<grid > 0 ? grid : n_items, kBTThreads, smem, st>>>(sd, items, n_items);
+        k_batch_fpb_bp<<<grid > 0 ? grid : n_items, kBTThreads, 0, st>>>(sd, items, n_items);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -2061,11 +2241,11 @@ cudaError_t launch_batch_fpb(const SolveDesc* sd, const int2* items, int n_items
     return cudaGetLastError();
 }
 
-cudaError_t batch_resident_ctas(int kernel, int threads, int* per_sm, size_t smem) {
+cudaError_t batch_resident_ctas(int kernel, int threads, int* per_sm) {
     switch (kernel) {
         case 0: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_proj, threads, 0);
         case 1: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_ray, threads, 0);
-        case 3: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_fpb_bp, threads, smem);
+        case 3: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_fpb_bp, threads, 0);
         default: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_bp, threads, 0);
     }
 }

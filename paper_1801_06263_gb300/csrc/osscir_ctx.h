@@ -59,17 +59,15 @@ struct osscir_ctx {
     float* fwd_w = nullptr;   // null: the forward projection stays on the fly
     int16_t* fwd_d = nullptr;
     uint32_t* bp_span = nullptr;
-    uint32_t* bp_row = nullptr;
-    float* bp_w = nullptr;   // null: the back-projection stays on the fly
-    uint16_t* bp_slot = nullptr;
-    uint32_t* bp_roff = nullptr;
-    int* bp_rays = nullptr;
+    uint32_t* bp_unit = nullptr;
+    float4* bp_w = nullptr;   // null: the back-projection stays on the fly
+    uint32_t* bp_slot = nullptr;
     float* bp_part = nullptr;
-    int bp_groups = 1, bp_chunk = 0, bp_nch = 0, bp_slots = 0;
+    int bp_groups = 1, bp_chunk = 0, bp_nch = 0, bp_wide = 0;
     size_t fp_bytes = 0;
     osscir::FpTables fp() const {
-        return osscir::FpTables{fwd_row, fwd_cnt, fwd_k0,  fwd_w,   fwd_d,     bp_span, bp_row, bp_w,
-                                bp_slot, bp_roff, bp_rays,   bp_part, bp_groups, bp_chunk, bp_nch, bp_slots};
+        return osscir::FpTables{fwd_row, fwd_cnt, fwd_k0,    fwd_w,    fwd_d,  bp_span,  bp_unit, bp_w,
+                                bp_slot, bp_part, bp_groups, bp_chunk, bp_nch, bp_wide};
     }
     const osscir::FpTables* fp_or_null() const { return fp_state == 1 ? &fp_tab : nullptr; }
     osscir::FpTables fp_tab{};

@@ -57,29 +57,32 @@ __device__ __forceinline__ float grid_plane(const GridF& G, int i) {
     return __fmaf_rn(static_cast<float>(i), G.h, G.x0);
 }
 
-// Per-ray record, 64 bytes per ray l = v * n_bins + b, stored as two arrays of
-// 32-byte halves in one allocation of 2 L RayRec: the weight half rec[l] and the
-// step half ray_steps(rec, L)[l].  Consecutive rays' halves are contiguous, so a
-// warp gathering the weight halves of neighbouring rays touches half as many
-// cache lines as with whole records.
+// Per-ray record, 68 bytes per ray l = v * n_bins + b, in one allocation
+// (ray_recs(L) RayRec): the weight halves rec[l], then the step's arrays
+// ray_steps(rec, L).  Consecutive rays are contiguous in each, so a warp gathering the
+// weight halves of neighbouring rays touches half as many cache lines as with whole
+// records, and the back-projection stages a view's bins by contiguous copies.
 //   rec[l].r0 = (bx, by, idx, idy)    foot point of the ray line nearest the origin and
 //                                     the reciprocal unit-direction components (inf if 0)
-//   rec[l].r1 = (ex, ey, b0, b1)      FP32 error bounds on t for x- and y-planes; b = alpha^T y'
-//   step.s0   = (b2, S00, S01, S02)   b and the block step matrix S = sum_w alpha_w alpha_w^T / |alpha_w|
-//   step.s1   = (S11, S12, S22, -)
+//   rec[l].r1 = (ex, ey, S22, -)      FP32 error bounds on t for x- and y-planes; S22 again
+//   s0[l]     = (b0, b1, b2, S00)     b = alpha^T y' and the block step matrix
+//   s1[l]     = (S01, S02, S11, S12)  S = sum_w alpha_w alpha_w^T / |alpha_w|
+//   s22[l]    = S22
 // r0 and r1.xy are written once per geometry; the rest once per MOCCA iteration.
 struct __align__(32) RayRec {
     float4 r0, r1;
 };
-struct __align__(32) RayStep {
-    float4 s0, s1;
+struct RaySteps {
+    float4* s0;
+    float4* s1;
+    float* s22;
 };
-__host__ __device__ __forceinline__ RayStep* ray_steps(RayRec* rec, int L) {
-    return reinterpret_cast<RayStep*>(rec + L);
+__host__ __device__ __forceinline__ RaySteps ray_steps(const RayRec* rec, int L) {
+    float4* s0 = reinterpret_cast<float4*>(const_cast<RayRec*>(rec) + L);
+    return RaySteps{s0, s0 + L, reinterpret_cast<float*>(s0 + 2 * (size_t)L)};
 }
-__host__ __device__ __forceinline__ const RayStep* ray_steps(const RayRec* rec, int L) {
-    return reinterpret_cast<const RayStep*>(rec + L);
-}
+// RayRecs to allocate for L rays.
+inline size_t ray_recs(int L) { return 2 * (size_t)L + ((size_t)L + 7) / 8; }
 
 // t(X) for the x-plane X along the unit direction from the foot point (mm).
 __device__ __forceinline__ float t_plane(float X, float b, float inv_d) {
@@ -317,27 +320,32 @@ struct GeomC {
     float margin_bins;       // candidate margin for the pixel-driven enumeration
 };
 
-// Candidate bin range of pixel (ix, iy) in a view: bins whose centre ray can cross
-// the pixel square (a superset of its shadow, in FP32 with a margin; x_weight decides).
-// With num = q . e_u and den = sid - q . e at the pixel's centre, a corner at
-// (+-h/2, +-h/2) from it moves beta by scale (dx (c num - s den) + dy (c den + s num)) /
-// (den den'), den' the corner's own den, so half the shadow's width is at most
-// scale h/2 (|c num - s den| + |c den + s num|) / (den min den').  One point and two
+// Bins whose centre ray can cross the box of half extents (hx, hy) around (X, Y) in a
+// view (a superset of its shadow, in FP32 with a margin; x_weight decides).  With
+// num = q . e_u and den = sid - q . e at the centre, a corner at (+-hx, +-hy) from it
+// moves beta by scale (dx (c num - s den) + dy (c den + s num)) / (den den'), den' the
+// corner's own den, so half the shadow's width is at most
+// scale (hx |c num - s den| + hy |c den + s num|) / (den min den').  One point and two
 // divisions instead of the four corners': about 25 instructions instead of 55 for
 // each of the pixel-views that the pixel-driven kernels visit; the bound is wider
-// than the shadow by a factor h / den at most (0.1 % at 256 x 256).
+// than the shadow by a factor h / den at most (0.1 % for a pixel at 256 x 256).
+__device__ __forceinline__ void box_bin_range(const GeomC& C, const ViewF& V, float X, float Y, float hx, float hy,
+                                              int& blo, int& bhi) {
+    const float num = fmaf(V.c, Y, -V.s * X), den = C.sid - fmaf(V.c, X, V.s * Y);
+    const float den_min = fmaxf(den - fmaf(hx, fabsf(V.c), hy * fabsf(V.s)), 1e-6f * den);
+    const float reach = fmaf(hx, fabsf(fmaf(V.c, num, -V.s * den)), hy * fabsf(fmaf(V.c, den, V.s * num)));
+    // __fdividef is within 2 ulp; the margin covers it
+    const float beta = fmaf(C.scale, __fdividef(num, den), C.mid);
+    const float half = fmaf(C.scale, __fdividef(reach, den * den_min), C.margin_bins);
+    blo = max(0, -sat_floor(half - beta));
+    bhi = min(C.n_bins - 1, sat_floor(beta + half));
+}
+
+// Candidate bin range of pixel (ix, iy) in a view.
 __device__ __forceinline__ void pixel_bin_range(const GeomC& C, const ViewF& V, int ix, int iy, int& blo,
                                                 int& bhi) {
     const float hh = 0.5f * C.grid.h;
-    const float X = grid_plane(C.grid, ix) + hh, Y = grid_plane(C.grid, iy) + hh;
-    const float num = fmaf(V.c, Y, -V.s * X), den = C.sid - fmaf(V.c, X, V.s * Y);
-    const float den_min = fmaxf(fmaf(-hh, fabsf(V.c) + fabsf(V.s), den), 1e-6f * den);
-    const float reach = fabsf(fmaf(V.c, num, -V.s * den)) + fabsf(fmaf(V.c, den, V.s * num));
-    // __fdividef is within 2 ulp; the margin covers it
-    const float beta = fmaf(C.scale, __fdividef(num, den), C.mid);
-    const float half = fmaf(C.scale * hh, __fdividef(reach, den * den_min), C.margin_bins);
-    blo = max(0, -sat_floor(half - beta));
-    bhi = min(C.n_bins - 1, sat_floor(beta + half));
+    box_bin_range(C, V, grid_plane(C.grid, ix) + hh, grid_plane(C.grid, iy) + hh, hh, hh, blo, bhi);
 }
 
 }  // namespace osscir

@@ -62,9 +62,11 @@ constexpr int kFwdThreads = 128;
 constexpr int kBpPixX = 2, kBpPixY = 32;              // MOCCA back-projection pixel tile (2 x 32: measured fastest)
 constexpr int kBpPix = kBpPixX * kBpPixY;                // also the plain back-projection's pixels per block
 constexpr int kBpMaxThreads = 512;                    // kBpPix x up to 8 view groups
-// Blocked back-projection table: a block is a tile of kBTX x kBTY pixels (one
-// per thread) and one view group; its views go in chunks of at most kBTMaxChunk.
-constexpr int kBTX = 16, kBTY = 16, kBTThreads = kBTX * kBTY, kBTMaxChunk = 16;
+// Blocked back-projection table: a block is a tile of kBTX x kBTY pixels (two, one
+// above the other, per thread) and one view group; its views go in chunks of at
+// most kBTMaxChunk.
+constexpr int kBTX = 16, kBTY = 16, kBTThreads = kBTX * kBTY / 2, kBTWarps = kBTThreads / 32, kBTMaxChunk = 16;
+constexpr int kBTSlots = 396;   // slots of a stage buffer (two of 36 bytes a slot: 28 KB, seven blocks per SM)
 inline int bt_tiles(int n) { return ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / kBTY); }
 
 // Footprint tables of one geometry: the pairs (l, k) of X with their weights,
@@ -79,16 +81,20 @@ inline int bt_tiles(int n) { return ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / 
 //   each rounded up to even.
 //   Back-projection (blocked): block b = t G + g (tile t, view group g of G =
 //   bp_groups); the group's views (the split of k_mocca_bp) in chunks of
-//   bp_chunk views, bp_nch chunks per group, entry e = b bp_nch + c.  bp_span
-//   [t n_views + u] = tlo | span << 16: the union of the tile's candidate bins in
-//   view u.  An entry's rays, view after view (ray (u, tlo + i)), are its stage
-//   slots: bp_rays[bp_roff[e] + slot], at most bp_slots of them.  The rows of
-//   warp w of entry e, bp_row[8 e + w] .. bp_row[8 e + w + 1] (an even number, so
-//   that a lane reads two rows with one load), are aligned per view: view u of
-//   the chunk takes as many rows as the warp's largest pair count in u.  Thread
-//   r's pairs (stage slot, weight) in the order of bp_pixel_sum sit at rows j of
-//   their view, (bp_slot, bp_w)[(row + j - j mod 2) 32 + 2 (r mod 32) + j mod 2];
-//   the rows a pixel does not fill hold the slot 0xffff.
+//   bp_chunk views, bp_nch chunks per group.  bp_span[t n_views + u] = tlo | span << 16:
+//   the bins that can meet the tile in view u.  A chunk's rays, view after view (ray
+//   (u, tlo + i)), are its stage slots, at most kBTSlots of them.  A thread has two
+//   pixels, (ix, iy) and (ix, iy + 1); in a view it has one entry per bin from the
+//   first to the last that meets either, with the weights of both (0 where the ray
+//   misses one).  The rows of a warp are aligned per view (view u takes as many rows
+//   as the warp's largest entry count in u, the other lanes' entries are zero
+//   weights) and a chunk's rows are rounded up to a multiple of four; a unit is four
+//   rows.  Warp w of block b has the units bp_unit[(b kBTWarps + w) nch + c] ..
+//   bp_unit[... + 1] in chunk c, contiguous over its chunks.  Unit q of lane r: weights
+//   bp_w[64 q + r] (two pixels of rows 0 and 1) and bp_w[64 q + 32 + r] (rows 2, 3);
+//   the rows' stage slots as four signed bytes bp_slot[32 q + r], each the step from the
+//   row before (from slot 0 at a chunk's start), or, where a step does not fit
+//   (bp_wide), as four 16-bit slots, bp_slot[64 q + 2 r] and + 1.
 //   bp_part: [G][9][P] scratch for the groups' channel sums.
 struct FpTables {
     const uint32_t* fwd_row;   // [n_views nbg + 1]
@@ -97,17 +103,12 @@ struct FpTables {
     const float* fwd_w;        // null: the forward projection is computed on the fly
     const int16_t* fwd_d;
     const uint32_t* bp_span;   // [bt_tiles(n) n_views]
-    const uint32_t* bp_row;    // [n_entries 8 + 1]
-    const float* bp_w;         // null: the back-projection is computed on the fly
-    const uint16_t* bp_slot;
-    const uint32_t* bp_roff;   // [n_entries + 1]
-    const int* bp_rays;
+    const uint32_t* bp_unit;   // [n_blocks kBTWarps nch + 1]
+    const float4* bp_w;        // null: the back-projection is computed on the fly
+    const uint32_t* bp_slot;
     float* bp_part;            // [bp_groups][9][P]
-    int bp_groups, bp_chunk, bp_nch, bp_slots;
+    int bp_groups, bp_chunk, bp_nch, bp_wide;
 };
-// Shared memory of the blocked back-projection's two stage buffers of `slots` slots.
-int fpb_stage_bytes(int slots);
-
 // View groups per pixel for the MOCCA back-projection: enough threads to fill
 // the GPU several times over, at most 8, and at least one view per group.
 inline int bp_view_groups(int n_pixels, int n_views) {
@@ -161,12 +162,21 @@ cudaError_t launch_xbar_columns(int n, float4* xbar, cudaStream_t st);
 // Fills fwd_w, fwd_d and fwd_k0; sets *bad if a pixel step does not fit in 16 bits.
 cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const uint32_t* fwd_row,
                                float* fwd_w, int16_t* fwd_d, int* fwd_k0, int* bad, cudaStream_t st);
-cudaError_t launch_fpb_span(const GeomC& C, const ViewF* views, uint32_t* span, cudaStream_t st);
-cudaError_t launch_fpb_count(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views, int G,
-                             int chunk, int nch, uint32_t* warp_rows, cudaStream_t st);
+// bp_span, and for each chunk size bt_size(i) the largest stage (slots) in most[i]
+// (zeroed before).
+constexpr int kBTSizes = 7;
+__host__ __device__ constexpr int bt_size(int i) {   // 1, 2, 4, 6, 8, 12, 16
+    return i < 3 ? 1 << i : (i == 3 ? 6 : (i == 4 ? 8 : (i == 5 ? 12 : kBTMaxChunk)));
+}
+cudaError_t launch_fpb_span(const GeomC& C, const ViewF* views, int G, uint32_t* span, int* most, cudaStream_t st);
+// The units of every (block, warp, chunk) at unit[1 + index], unit[0] = 0 (a prefix sum
+// of the former makes bp_unit); *wide set if a slot step does not fit a signed byte.
+cudaError_t launch_fpb_count(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
+                             const FpTables& T, uint32_t* unit, int* wide, cudaStream_t st);
+// In-place inclusive prefix sum of v[0 .. n) modulo 2^32 (one block); *total the 64-bit sum.
+cudaError_t launch_scan(uint32_t* v, size_t n, unsigned long long* total, cudaStream_t st);
 cudaError_t launch_fpb_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
-                            const uint32_t* span, int G, int chunk, int nch, const uint32_t* bp_row, float* bp_w,
-                            uint16_t* bp_slot, cudaStream_t st);
+                            const FpTables& T, float4* bp_w, uint32_t* bp_slot, cudaStream_t st);
 cudaError_t launch_mocca_apply(const GeomC& C, const StepParams& P, const SolveD& D, const float* chan,
                                cudaStream_t st);
 
@@ -215,12 +225,11 @@ cudaError_t launch_batch_bp(const SolveDesc* sd, const int2* items, int n_items,
                             cudaStream_t st);
 cudaError_t launch_batch_dtpl(const SolveDesc* sd, int n_solves, cudaStream_t st);
 // Back-projection of solves with footprint tables: items (solve, table block),
-// then fin_items (solve, block of 256 pixels) for the group sums and a7; smem:
-// the largest solve's two stage buffers (fpb_stage_bytes).
+// then fin_items (solve, block of 256 pixels) for the group sums and a7.
 cudaError_t launch_batch_fpb(const SolveDesc* sd, const int2* items, int n_items, const int2* fin_items,
-                             int n_fin, int grid, size_t smem, cudaStream_t st);
+                             int n_fin, int grid, cudaStream_t st);
 // Resident CTAs per SM of a batched kernel (0 projection, 1 ray, 2 back-projection
-// on the fly, 3 back-projection from tables with smem bytes of dynamic shared memory).
-cudaError_t batch_resident_ctas(int kernel, int threads, int* per_sm, size_t smem = 0);
+// on the fly, 3 back-projection from tables).
+cudaError_t batch_resident_ctas(int kernel, int threads, int* per_sm);
 
 }  // namespace osscir
