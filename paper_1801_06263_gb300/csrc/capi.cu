@@ -53,7 +53,7 @@ void free_ctx(osscir_ctx* h) {
     if (h->join) cudaEventDestroy(h->join);
     void* ptrs[] = {h->rec,     h->r64,    h->views,     h->chord,    h->exc_off,    h->exc_ent,  h->s4,
                     h->N4,      h->mu,     h->mu_in,     h->g,        h->c,          h->y,        h->x,
-                    h->xbar,    h->xo,     h->dtpl_part, h->dtpl_out, h->bad_counts, h->model,    h->fwd_row,
+                    h->xbar,    h->xo,     h->dtpl_part, h->dtpl_out, h->bad_counts, h->model,    h->fwd_unit,
                     h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit, h->bp_w,
                     h->bp_slot, h->bp_part};
     for (void* p : ptrs)
@@ -345,11 +345,11 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
 }
 
 void free_tables(osscir_ctx* h) {
-    void* ptrs[] = {h->fwd_row, h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit,
+    void* ptrs[] = {h->fwd_unit, h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit,
                     h->bp_w,    h->bp_slot, h->bp_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    h->fwd_row = nullptr;
+    h->fwd_unit = nullptr;
     h->fwd_cnt = nullptr;
     h->fwd_k0 = nullptr;
     h->fwd_w = nullptr;
@@ -361,20 +361,6 @@ void free_tables(osscir_ctx* h) {
     h->bp_part = nullptr;
     h->bytes -= h->fp_bytes;
     h->fp_bytes = 0;
-}
-
-// Device array of the prefix sums of n counts (in place on the host copy), with
-// its total appended; false if the total does not fit 32 bits.
-bool prefix_rows(std::vector<uint32_t>& v, size_t n) {
-    uint64_t run = 0;
-    for (size_t i = 0; i < n; ++i) {
-        const uint64_t c = v[i];
-        v[i] = (uint32_t)run;
-        run += c;
-    }
-    if (run > 0xffffffffull) return false;
-    v[n] = (uint32_t)run;
-    return true;
 }
 
 // Build the footprint tables (FpTables) once per context, before the first
@@ -407,50 +393,37 @@ osscir_status build_tables(osscir_ctx* h) {
     } while (0)
     // forward: per-ray counts and per-warp rows, then the pairs
     CKT(dalloc(&h->fwd_cnt, (size_t)h->L));
-    CKT(dalloc(&h->fwd_row, n_fw + 1));
-    CKT(launch_fp_fwd_count(C, h->exc(), h->rec, h->fwd_cnt, h->fwd_row, st));
-    std::vector<uint32_t> rows(n_fw + 1, 0);
-    CKT(cudaMemcpyAsync(rows.data(), h->fwd_row, sizeof(uint32_t) * n_fw, cudaMemcpyDeviceToHost, st));
-    CKT(cudaStreamSynchronize(st));
-    for (size_t i = 0; i < n_fw; ++i) rows[i] = (rows[i] + 1) & ~1u;   // even: entries are read two at a time
-    if (!prefix_rows(rows, n_fw)) return fail(cudaErrorMemoryAllocation);
-    CKT(cudaMemcpyAsync(h->fwd_row, rows.data(), sizeof(uint32_t) * (n_fw + 1), cudaMemcpyHostToDevice, st));
-    CKT(dalloc(&h->fwd_w, (size_t)rows[n_fw] * 32));
-    CKT(dalloc(&h->fwd_d, (size_t)rows[n_fw] * 32));
-    CKT(dalloc(&h->fwd_k0, (size_t)h->L));
-    {
-        int* bad = nullptr;   // a pixel step outside 16 bits: keep the on-the-fly projections
-        CKT(dalloc(&bad, 1));
-        int bad_h = 0;
-        cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), st);
-        if (e == cudaSuccess) e = launch_fp_fwd_fill(C, h->exc(), h->rec, h->fwd_row, h->fwd_w, h->fwd_d, h->fwd_k0,
-                                                     bad, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bad_h, bad, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        cudaFree(bad);
-        h->bytes -= sizeof(int);
-        CKT(e);
-        if (bad_h) return fail(cudaErrorMemoryAllocation);
-    }
-    // back-projection (blocked): per tile and view the bins that can meet it; the chunk
-    // size (views per staged chunk) whose two stage buffers fit; the units of each
-    // (block, warp, chunk) and their prefix sum; then the entries
-    const int n_t = bt_tiles(C.grid.n), per = (C.n_views + G - 1) / G;
-    CKT(dalloc(&h->bp_span, (size_t)n_t * C.n_views));
+    CKT(dalloc(&h->fwd_unit, n_fw + 1));
     struct {
-        unsigned long long total;
-        int most[kBTSizes], wide;
+        unsigned long long total, fwd_total;
+        int most[kBTSizes], wide, bad;   // bad: a pixel step outside 16 bits
     } stat{};
-    int* stat_d = nullptr;
-    CKT(dalloc(&stat_d, sizeof stat / sizeof(int)));
-    unsigned long long* total_d = reinterpret_cast<unsigned long long*>(stat_d);
-    cudaError_t e = cudaMemsetAsync(stat_d, 0, sizeof stat, st);
+    char* stat_d = nullptr;
+    CKT(dalloc(&stat_d, sizeof stat));
+    auto dev = [&](auto* field) {   // where the field lies on the device
+        return reinterpret_cast<decltype(field)>(stat_d + (reinterpret_cast<char*>(field) - reinterpret_cast<char*>(&stat)));
+    };
     auto read_stat = [&]() {
         cudaError_t r = cudaMemcpyAsync(&stat, stat_d, sizeof stat, cudaMemcpyDeviceToHost, st);
         return r != cudaSuccess ? r : cudaStreamSynchronize(st);
     };
-    if (e == cudaSuccess) e = launch_fpb_span(C, h->views, G, h->bp_span, stat_d + 2, st);
+    cudaError_t e = cudaMemsetAsync(stat_d, 0, sizeof stat, st);
+    if (e == cudaSuccess) e = launch_fp_fwd_count(C, h->exc(), h->rec, h->fwd_cnt, h->fwd_unit, st);
+    if (e == cudaSuccess) e = launch_scan(h->fwd_unit + 1, n_fw, dev(&stat.fwd_total), st);
+    // back-projection (blocked): per tile and view the bins that can meet it; the chunk
+    // size (views per staged chunk) whose two stage buffers fit; the units of each
+    // (block, warp, chunk) and their prefix sum; then the entries
+    const int n_t = bt_tiles(C.grid.n), per = (C.n_views + G - 1) / G;
+    if (e == cudaSuccess) e = dalloc(&h->bp_span, (size_t)n_t * C.n_views);
+    if (e == cudaSuccess) e = launch_fpb_span(C, h->views, G, h->bp_span, dev(&stat.most[0]), st);
     if (e == cudaSuccess) e = read_stat();
+    // forward: the pairs; one more unit than the table has (it is loaded ahead)
+    if (e == cudaSuccess && stat.fwd_total > 0xffffffffull) e = cudaErrorMemoryAllocation;
+    if (e == cudaSuccess) e = dalloc(&h->fwd_w, ((size_t)stat.fwd_total + 1) * 128);
+    if (e == cudaSuccess) e = dalloc(&h->fwd_d, ((size_t)stat.fwd_total + 1) * 128);
+    if (e == cudaSuccess) e = dalloc(&h->fwd_k0, (size_t)h->L);
+    if (e == cudaSuccess)
+        e = launch_fp_fwd_fill(C, h->exc(), h->rec, h->fwd_unit, h->fwd_w, h->fwd_d, h->fwd_k0, dev(&stat.bad), st);
     int chunk = 0;
     for (int i = kBTSizes - 1; i >= 0 && !chunk && C.n_bins <= 65535; --i)   // bp_span holds a bin in 16 bits
         if (stat.most[i] <= kBTSlots) chunk = bt_size(i);
@@ -461,8 +434,8 @@ osscir_status build_tables(osscir_ctx* h) {
         const size_t n_u = (size_t)n_t * G * kBTWarps * h->bp_nch;
         e = dalloc(&h->bp_unit, n_u + 1);
         if (e == cudaSuccess)
-            e = launch_fpb_count(C, h->exc(), h->rec, h->views, h->fp(), h->bp_unit, stat_d + 2 + kBTSizes, st);
-        if (e == cudaSuccess) e = launch_scan(h->bp_unit + 1, n_u, total_d, st);
+            e = launch_fpb_count(C, h->exc(), h->rec, h->views, h->fp(), h->bp_unit, dev(&stat.wide), st);
+        if (e == cudaSuccess) e = launch_scan(h->bp_unit + 1, n_u, dev(&stat.total), st);
         if (e == cudaSuccess) e = read_stat();
         if (e == cudaSuccess && stat.total > 0xffffffffull) e = cudaErrorMemoryAllocation;
         h->bp_wide = stat.wide;
@@ -471,6 +444,8 @@ osscir_status build_tables(osscir_ctx* h) {
         if (e == cudaSuccess) e = dalloc(&h->bp_w, ((size_t)stat.total + 1) * 64);   // one more unit: it is loaded ahead
         if (e == cudaSuccess) e = launch_fpb_fill(C, h->exc(), h->rec, h->views, h->fp(), h->bp_w, h->bp_slot, st);
     }
+    if (e == cudaSuccess) e = read_stat();
+    if (e == cudaSuccess && stat.bad) e = cudaErrorMemoryAllocation;
     cudaFree(stat_d);
     h->bytes -= sizeof stat;
     CKT(e);

@@ -16,6 +16,8 @@
 //       P_k = sum_l X_lk S_l (so T^-1_k = P_k / lambda, the m-block SPC), the
 //       3x3 solve (double-float), the primal step (optionally onto a box) and the
 //       extrapolation xbar' = 2 x' - x.
+#include <type_traits>
+
 #include "osscir_dfl.cuh"
 #include "osscir_internal.cuh"
 #include "osscir_launch.h"
@@ -135,6 +137,11 @@ __device__ __forceinline__ uint2 ld_stream(const uint2* p) {
     uint2 u;
     asm("ld.global.nc.L1::no_allocate.v2.b32 {%0, %1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(p));
     return u;
+}
+
+// Bytes (a multiple of 16, from a 16-byte boundary) on their way from HBM to L2.
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // Half of a ray record (32 bytes, 32-byte aligned) in one 256-bit load.
@@ -1298,9 +1305,9 @@ __global__ void k_mocca_apply(GeomC C, StepParams P, SolveD D, const float* __re
 // for bit the same.  See FpTables for the layout.
 
 // Forward table, pass 1: the footprint size of every ray, and per warp (view,
-// 32-bin group) the largest one: its number of slot rows.
+// 32-bin group) w the units of four pairs of the largest one, at unit[1 + w].
 __global__ void __launch_bounds__(kFwdThreads) k_fp_fwd_count(GeomC C, ExcTable E, const RayRec* rec, int* cnt,
-                                                              uint32_t* warp_rows) {
+                                                              uint32_t* unit) {
     const int l = ray_of_thread(C);
     int n = 0;
     if (l >= 0) {
@@ -1310,11 +1317,13 @@ __global__ void __launch_bounds__(kFwdThreads) k_fp_fwd_count(GeomC C, ExcTable 
     }
     n = __reduce_max_sync(0xffffffffu, n);
     const int v = warp_view(blockIdx.y, kFwdThreads / 32);
-    if ((threadIdx.x & 31) == 0 && v < C.n_views) warp_rows[v * ((C.n_bins + 31) >> 5) + blockIdx.x] = (uint32_t)n;
+    if ((threadIdx.x & 31) == 0 && v < C.n_views)
+        unit[1 + v * ((C.n_bins + 31) >> 5) + blockIdx.x] = (uint32_t)((n + 3) / 4);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) unit[0] = 0;
 }
 
 // Forward table, pass 2: lane r of warp w writes its j-th pair (weight, pixel
-// step) in visiting order, two per slot row from fwd_row[w] (see FpTables).
+// step) in visiting order, four per unit from fwd_unit[w] (see FpTables).
 // Each ray's pixels index the xbar copy in which the warp's gathers at one
 // table row are close.  The lanes advance from their first pixels at about the
 // same pace along the slabs, so what matters is the image edge a ray enters
@@ -1325,104 +1334,111 @@ __global__ void __launch_bounds__(kFwdThreads) k_fp_fwd_count(GeomC C, ExcTable 
 // own first pixel: 7.8 distinct 128-byte lines per warp gather at 256x256,
 // against 12.0 when the warp chose by the rays' direction.
 __global__ void __launch_bounds__(kFwdThreads) k_fp_fwd_fill(GeomC C, ExcTable E, const RayRec* rec,
-                                                             const uint32_t* __restrict__ fwd_row, float* fwd_w,
+                                                             const uint32_t* __restrict__ fwd_unit, float* fwd_w,
                                                              int16_t* fwd_d, int* fwd_k0, int* bad) {
     const int l = ray_of_thread(C);
     if (l < 0) return;
     const int v = warp_view(blockIdx.y, kFwdThreads / 32);
-    const size_t row = fwd_row[v * ((C.n_bins + 31) >> 5) + blockIdx.x];
+    const size_t q0 = fwd_unit[v * ((C.n_bins + 31) >> 5) + blockIdx.x];
     const int lane = threadIdx.x & 31, n = C.grid.n;
     const float4 r0 = rec[l].r0, r1 = rec[l].r1;
     int j = 0, prev = -1;
     bool col = false;
+    auto put = [&](int d, float w) {
+        const size_t at = ((q0 + (j >> 2)) * 32 + lane) * 4 + (j & 3);
+        fwd_w[at] = w;
+        fwd_d[at] = (int16_t)d;
+        ++j;
+    };
     ray_pixels(C, E, r0, r1.x, r1.y, l, [&](int kr, float w) {
         if (j == 0) col = kr % n == 0 || kr % n == n - 1;   // entered through a left or right edge
         const int k = col ? n * n + (kr % n) * n + kr / n : kr;
-        const size_t at = (row + (j & ~1)) * 32 + 2 * lane + (j & 1);
         if (j == 0) {
             fwd_k0[l] = k;
             prev = k;
         }
         const int d = k - prev;
         if (d < -32768 || d > 32767) *bad = 1;
-        fwd_w[at] = w;
-        fwd_d[at] = (int16_t)d;
+        put(d, w);
         prev = k;
-        ++j;
     });
     if (j == 0) fwd_k0[l] = 0;
+    while (j & 3) put(0, 0.0f);   // the rest of the ray's last unit
 }
+
+// One unit of a lane: four weights and the four 16-bit pixel steps.
+struct FwdUnit {
+    float4 w;
+    int2 d;
+};
+__device__ __forceinline__ FwdUnit ld_fwd(const float4* w, const int2* d) { return FwdUnit{__ldg(w), __ldg(d)}; }
 
 // a1 from the forward table for ray l of warp wi = v nbg + bx: the same line sums
-// as proj_ray, in the same order.  The table is read four entries (two loads of
-// two) at a time, the next four loaded while the current four's gathers of xbar
-// are added, so a table load is always in flight.
+// as proj_ray, in the same order (an FP32 partial over kFold pixels folded into the
+// total; the zero weights that fill a ray's last unit add nothing).  UN units go per
+// trip of the main loop, so that their 4 UN gathers of xbar are in flight together,
+// and the next unit's entries are loaded while the current one's are added (one unit
+// past the table's end is allocated for that).  The pixel indices come from one 16-bit
+// dot product each: 9 instructions a pair instead of 24.
+// What bounds it: at 256 x 256 the L1 data pipe (71 % of its wavefronts; a warp gather
+// takes one for each of the 7.8 lines it touches), at 512 x 512 that and HBM; a grid of
+// few blocks the gathers' latency.
+template <int UN>
 __device__ __forceinline__ void fp_proj_ray(const FpTables& T, const SolveD& D, int l, int wi) {
-    const int lane = threadIdx.x & 31;
-    const size_t base = (size_t)T.fwd_row[wi] * 32;
-    const float2* pw = reinterpret_cast<const float2*>(T.fwd_w + base) + lane;
-    const short2* pd = reinterpret_cast<const short2*>(T.fwd_d + base) + lane;
-    const int n = __ldg(T.fwd_cnt + l);
+    const size_t at = (size_t)__ldg(T.fwd_unit + wi) * 32 + (threadIdx.x & 31);
+    const float4* wp = reinterpret_cast<const float4*>(T.fwd_w) + at;
+    const int2* dp = reinterpret_cast<const int2*>(T.fwd_d) + at;
+    int left = (__ldg(T.fwd_cnt + l) + 3) >> 2;   // the ray's units
     int k = __ldg(T.fwd_k0 + l);
-    LineSum acc;
-    int j = 0;
-    if (n >= 4) {
-        float2 w[2];
-        short2 d[2];
+    float p0 = 0.f, p1 = 0.f, p2 = 0.f, t0 = 0.f, t1 = 0.f, t2 = 0.f;
+    auto unit = [&](const FwdUnit& u) {
+        const int ka = __dp2a_lo(u.d.x, 0x0001, k), kb = __dp2a_lo(u.d.x, 0x0101, k);
+        const int kc = __dp2a_lo(u.d.y, 0x0001, kb), kd = __dp2a_lo(u.d.y, 0x0101, kb);
+        const float4 a = __ldg(D.xbar + ka), b = __ldg(D.xbar + kb), c = __ldg(D.xbar + kc), d = __ldg(D.xbar + kd);
+        k = kd;
+        p0 = fmaf(u.w.x, a.x, p0), p1 = fmaf(u.w.x, a.y, p1), p2 = fmaf(u.w.x, a.z, p2);
+        p0 = fmaf(u.w.y, b.x, p0), p1 = fmaf(u.w.y, b.y, p1), p2 = fmaf(u.w.y, b.z, p2);
+        p0 = fmaf(u.w.z, c.x, p0), p1 = fmaf(u.w.z, c.y, p1), p2 = fmaf(u.w.z, c.z, p2);
+        p0 = fmaf(u.w.w, d.x, p0), p1 = fmaf(u.w.w, d.y, p1), p2 = fmaf(u.w.w, d.z, p2);
+    };
+    static_assert(kFold == 16, "four units per fold");
+    if (left > 0) {
+        FwdUnit next = ld_fwd(wp, dp);
+        auto units = [&](auto count) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            w[u] = __ldg(pw + 32 * u);
-            d[u] = __ldg(pd + 32 * u);
-        }
-        for (; j + 3 < n; j += 4) {
-            pw += 64;
-            pd += 64;
-            float2 wn[2];
-            short2 dn[2];
-            const bool more = j + 7 < n;
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                wn[u] = more ? __ldg(pw + 32 * u) : make_float2(0.f, 0.f);
-                dn[u] = more ? __ldg(pd + 32 * u) : make_short2(0, 0);
+            for (int i = 0; i < decltype(count)::value; ++i) {
+                const FwdUnit u = next;
+                wp += 32;
+                dp += 32;
+                next = ld_fwd(wp, dp);
+                unit(u);
+                if (i % 4 == 3) {
+                    t0 += p0, t1 += p1, t2 += p2;
+                    p0 = p1 = p2 = 0.f;
+                }
             }
-            int kk[4];
-            kk[0] = k + d[0].x;
-            kk[1] = kk[0] + d[0].y;
-            kk[2] = kk[1] + d[1].x;
-            kk[3] = kk[2] + d[1].y;
-            k = kk[3];
-            float4 x[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = __ldg(D.xbar + kk[u]);
-            acc.add(w[0].x, x[0]);
-            acc.add(w[0].y, x[1]);
-            acc.add(w[1].x, x[2]);
-            acc.add(w[1].y, x[3]);
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                w[u] = wn[u];
-                d[u] = dn[u];
-            }
-        }
+            left -= decltype(count)::value;
+        };
+#pragma unroll 1
+        while (left >= UN) units(std::integral_constant<int, UN>());
+        if (UN > 4 && left >= 4) units(std::integral_constant<int, 4>());
+        if (left & 2) units(std::integral_constant<int, 2>());
+        if (left > 0) units(std::integral_constant<int, 1>());
     }
-    for (; j < n; j += 2, pw += 32, pd += 32) {
-        const float2 w = __ldg(pw);
-        const short2 d = __ldg(pd);
-        k += d.x;
-        acc.add(w.x, __ldg(D.xbar + k));
-        if (j + 1 < n) {
-            k += d.y;
-            acc.add(w.y, __ldg(D.xbar + k));
-        }
-    }
-    const float4 gs = acc.sum();
-    D.g[l] = make_float4(gs.x, gs.y, gs.z, 0.f);
+    D.g[l] = make_float4(t0 + p0, t1 + p1, t2 + p2, 0.f);
 }
 
-__global__ void __launch_bounds__(kFwdThreads, 8) k_fp_proj(GeomC C, FpTables T, SolveD D, int v0, int v1) {
+// Loads in flight count for more than resident warps: with four units per trip and the
+// registers for it 86 us at 256 x 256 (six resident blocks 93, eight 95, ten 99; 109
+// before).  Eight units per trip take a 64 x 64 image's 128 blocks 15 instead of
+// 18.5 us and 630 blocks of 300 x 300 56 instead of 63 us, but 256 x 256's 2048 blocks
+// 98 us: kFwdFewBlocks lies between.
+constexpr unsigned kFwdFewBlocks = 6 * 152;   // six blocks per SM
+template <int UN>
+__global__ void __launch_bounds__(kFwdThreads, UN > 4 ? 3 : 4) k_fp_proj(GeomC C, FpTables T, SolveD D, int v0, int v1) {
     const int bx = centre_out(blockIdx.y, gridDim.y);
     const int l = ray_in_views(C, bx, blockIdx.x, kFwdThreads / 32, v0, v1);
-    if (l >= 0) fp_proj_ray(T, D, l, (l / C.n_bins) * ((C.n_bins + 31) >> 5) + bx);
+    if (l >= 0) fp_proj_ray<UN>(T, D, l, (l / C.n_bins) * ((C.n_bins + 31) >> 5) + bx);
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t smem, const void* gmem) {
@@ -1674,11 +1690,6 @@ __device__ __forceinline__ void stage_views(const GeomC& C, const RaySteps& step
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// Bytes (a multiple of 16, from a 16-byte boundary) on their way from HBM to L2.
-__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // One unit of a lane: four rows' weights of its two pixels and their stage slots.
@@ -1969,7 +1980,7 @@ __global__ void __launch_bounds__(kBatchProjMaxThreads) k_batch_proj(const Solve
         const int bx = centre_out(w.y / nby, nbx);
         const int l = ray_at(C, bx, w.y % nby, vb);
         if (l >= 0) {
-            if (d.T.fwd_w) fp_proj_ray(d.T, d.D, l, (l / C.n_bins) * nbx + bx);   // the solve's table
+            if (d.T.fwd_w) fp_proj_ray<4>(d.T, d.D, l, (l / C.n_bins) * nbx + bx);   // the solve's table
             else proj_ray(C, d.E, d.rec, d.D, l);
         }
     }
@@ -2088,7 +2099,8 @@ cudaError_t launch_mocca_proj(const GeomC& C, const ExcTable& E, const RayRec* r
                               cudaStream_t st, int v0, int v1, const FpTables* T) {
     if (v1 < 0) v1 = C.n_views;
     const dim3 fg = fwd_grid(C.n_bins, v1 - v0);
-    if (T) k_fp_proj<<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, *T, D, v0, v1);
+    if (T && fg.x * fg.y <= kFwdFewBlocks) k_fp_proj<8><<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, *T, D, v0, v1);
+    else if (T) k_fp_proj<4><<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, *T, D, v0, v1);
     else k_mocca_proj<<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, E, rec, D, v0, v1);
     return cudaGetLastError();
 }
@@ -2156,14 +2168,14 @@ cudaError_t launch_xbar_columns(int n, float4* xbar, cudaStream_t st) {
 }
 
 cudaError_t launch_fp_fwd_count(const GeomC& C, const ExcTable& E, const RayRec* rec, int* cnt,
-                                uint32_t* warp_rows, cudaStream_t st) {
-    k_fp_fwd_count<<<fwd_grid(C.n_bins, C.n_views), kFwdThreads, 0, st>>>(C, E, rec, cnt, warp_rows);
+                                uint32_t* unit, cudaStream_t st) {
+    k_fp_fwd_count<<<fwd_grid(C.n_bins, C.n_views), kFwdThreads, 0, st>>>(C, E, rec, cnt, unit);
     return cudaGetLastError();
 }
 
-cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const uint32_t* fwd_row,
+cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const uint32_t* fwd_unit,
                                float* fwd_w, int16_t* fwd_d, int* fwd_k0, int* bad, cudaStream_t st) {
-    k_fp_fwd_fill<<<fwd_grid(C.n_bins, C.n_views), kFwdThreads, 0, st>>>(C, E, rec, fwd_row, fwd_w, fwd_d, fwd_k0,
+    k_fp_fwd_fill<<<fwd_grid(C.n_bins, C.n_views), kFwdThreads, 0, st>>>(C, E, rec, fwd_unit, fwd_w, fwd_d, fwd_k0,
                                                                          bad);
     return cudaGetLastError();
 }

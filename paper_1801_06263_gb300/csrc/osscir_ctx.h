@@ -53,7 +53,7 @@ struct osscir_ctx {
     float4* model = nullptr;
     // footprint tables (built before the first plain iteration; see FpTables)
     int fp_state = 0;   // 0 not built yet, 1 built, -1 not used (no room on the device)
-    uint32_t* fwd_row = nullptr;
+    uint32_t* fwd_unit = nullptr;
     int* fwd_cnt = nullptr;
     int* fwd_k0 = nullptr;
     float* fwd_w = nullptr;   // null: the forward projection stays on the fly
@@ -66,7 +66,7 @@ struct osscir_ctx {
     int bp_groups = 1, bp_chunk = 0, bp_nch = 0, bp_wide = 0;
     size_t fp_bytes = 0;
     osscir::FpTables fp() const {
-        return osscir::FpTables{fwd_row, fwd_cnt, fwd_k0,    fwd_w,    fwd_d,  bp_span,  bp_unit, bp_w,
+        return osscir::FpTables{fwd_unit, fwd_cnt, fwd_k0,    fwd_w,    fwd_d,  bp_span,  bp_unit, bp_w,
                                 bp_slot, bp_part, bp_groups, bp_chunk, bp_nch, bp_wide};
     }
     const osscir::FpTables* fp_or_null() const { return fp_state == 1 ? &fp_tab : nullptr; }

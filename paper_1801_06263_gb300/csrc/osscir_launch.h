@@ -73,12 +73,12 @@ inline int bt_tiles(int n) { return ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / 
 // in the order each projector visits them.
 //   Forward (ray-major): warp w = (view v, 32-bin group bx), w = v nbg + bx with
 //   nbg = ceil(n_bins / 32), lane r = bin 32 bx + r.  Ray l has fwd_cnt[l] pairs
-//   in the visiting order of ray_weights; its j-th pair is the weight fwd_w[i]
-//   and the pixel k_j = fwd_k0[l] + sum_{i <= j} fwd_d[i] (fwd_d: the 16-bit step
-//   from the previous pixel, 0 for the first), at i = (fwd_row[w] + j - j mod 2)
-//   32 + 2 r + j mod 2: two pairs side by side, so a lane reads two with one load
-//   (6 bytes a pair).  fwd_row is the prefix sum of the warps' largest counts,
-//   each rounded up to even.
+//   in the visiting order of ray_weights, four to a unit: its j-th pair is the weight
+//   fwd_w[i] and the pixel k_j = fwd_k0[l] + sum_{i <= j} fwd_d[i] (fwd_d: the 16-bit
+//   step from the previous pixel, 0 for the first), at
+//   i = ((fwd_unit[w] + j / 4) 32 + r) 4 + j mod 4: a lane reads a unit with one
+//   16-byte and one 8-byte load (6 bytes a pair).  A ray's last unit is filled up with
+//   zero weights and steps.  fwd_unit is the prefix sum of the warps' largest units.
 //   Back-projection (blocked): block b = t G + g (tile t, view group g of G =
 //   bp_groups); the group's views (the split of k_mocca_bp) in chunks of
 //   bp_chunk views, bp_nch chunks per group.  bp_span[t n_views + u] = tlo | span << 16:
@@ -97,7 +97,7 @@ inline int bt_tiles(int n) { return ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / 
 //   (bp_wide), as four 16-bit slots, bp_slot[64 q + 2 r] and + 1.
 //   bp_part: [G][9][P] scratch for the groups' channel sums.
 struct FpTables {
-    const uint32_t* fwd_row;   // [n_views nbg + 1]
+    const uint32_t* fwd_unit;  // [n_views nbg + 1]
     const int* fwd_cnt;        // [L]
     const int* fwd_k0;         // [L] first pixel of each ray
     const float* fwd_w;        // null: the forward projection is computed on the fly
@@ -153,14 +153,14 @@ cudaError_t launch_dtpl_reduce(const double* part, int n, double* out, cudaStrea
 cudaError_t launch_mocca_bp_partial(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
                                     const StepParams& P, const SolveD& D, int v0, int v1, float* chan,
                                     cudaStream_t st, const FpTables* T = nullptr);
-// Footprint table construction: counts (forward: per ray, and per warp the slot
-// rows; back-projection: slot rows per entry), then the fills from the row offsets.
+// Footprint table construction: counts (forward: per ray, and per warp w its units at
+// unit[1 + w], unit[0] = 0; back-projection: units), their prefix sums, then the fills.
 cudaError_t launch_fp_fwd_count(const GeomC& C, const ExcTable& E, const RayRec* rec, int* cnt,
-                                uint32_t* warp_rows, cudaStream_t st);
+                                uint32_t* unit, cudaStream_t st);
 // Writes the column-major copy of xbar ([2P]: P + ix n + iy) from its row-major half.
 cudaError_t launch_xbar_columns(int n, float4* xbar, cudaStream_t st);
 // Fills fwd_w, fwd_d and fwd_k0; sets *bad if a pixel step does not fit in 16 bits.
-cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const uint32_t* fwd_row,
+cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const uint32_t* fwd_unit,
                                float* fwd_w, int16_t* fwd_d, int* fwd_k0, int* bad, cudaStream_t st);
 // bp_span, and for each chunk size bt_size(i) the largest stage (slots) in most[i]
 // (zeroed before).

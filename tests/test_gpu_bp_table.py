@@ -1,7 +1,8 @@
 """The blocked back-projection table (csrc/mocca.cu) at the sizes where it can go wrong:
 images that are no multiple of a tile or of a pixel pair, fewer views than view groups,
 16-bit slots (a tile seen by more bins than a signed byte steps over), a chunk that ends
-mid-group and view ranges that straddle chunks.  Two iterations against the FP64 oracle
+mid-group, view ranges that straddle chunks, and a grid of many blocks whose rays meet a
+few pixels (the forward table's four-unit form; the other images take the eight-unit one).  Two iterations against the FP64 oracle
 (relative L2 1e-5: a few FP32 roundings of sums whose pixels the double-float step
 solves), and the sums over split view ranges against the whole's (1e-6: another order
 of the same FP32 additions)."""
@@ -14,7 +15,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,views,bins", [(33, 45, 256), (16, 24, 24), (50, 61, 77), (47, 130, 64), (1, 40, 33)])
+@pytest.mark.parametrize("n,views,bins", [(33, 45, 256), (16, 24, 24), (50, 61, 77), (47, 130, 64), (1, 40, 33), (5, 1024, 130)])
 def test_table_backprojection(orc, n, views, bins):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
