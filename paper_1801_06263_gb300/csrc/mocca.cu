@@ -989,10 +989,10 @@ __device__ __forceinline__ bool box_step3(const dfl (&p)[6], const dfl (&t)[3], 
     for (int i = 0; i < 3; ++i) {
         const int j = (i + 1) % 3, k = (i + 2) % 3;
         // (x_j - t_j, x_k - t_k) = d_i (wj, wk)
-        const dfl qji = p[at[j][i]], qjk = p[at[j][k]], r = df_rcp(p[at[j][j]]), l = df_mul(qjk, r);
+        const dfl qji = p[at[j][i]], qjk = p[at[j][k]], r = df_rcp_fma(p[at[j][j]]), l = df_mul(qjk, r);
         const dfl schur = df_sub(p[at[k][k]], df_mul(l, qjk));
         if (!(schur.hi > 0.0f)) return false;
-        const dfl wk = df_mul(df_sub(df_mul(l, qji), p[at[k][i]]), df_rcp(schur));
+        const dfl wk = df_mul(df_sub(df_mul(l, qji), p[at[k][i]]), df_rcp_fma(schur));
         const dfl wj = df_neg(df_mul(df_add(qji, df_mul(qjk, wk)), r));
 #pragma unroll 1
         for (int side = 0; side < 2; ++side) {
@@ -1011,7 +1011,7 @@ __device__ __forceinline__ bool box_step3(const dfl (&p)[6], const dfl (&t)[3], 
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int i = (k + 1) % 3, j = (k + 2) % 3;
-        const dfl qki = p[at[k][i]], qkj = p[at[k][j]], r = df_rcp(p[at[k][k]]), li = df_mul(qki, r), lj = df_mul(qkj, r);
+        const dfl qki = p[at[k][i]], qkj = p[at[k][j]], r = df_rcp_fma(p[at[k][k]]), li = df_mul(qki, r), lj = df_mul(qkj, r);
         const dfl sii = df_sub(p[at[i][i]], df_mul(li, qki)), sjj = df_sub(p[at[j][j]], df_mul(lj, qkj));
         const dfl sij = df_sub(p[at[i][j]], df_mul(li, qkj));
 #pragma unroll 1
@@ -1188,16 +1188,36 @@ __device__ __forceinline__ void bp_finish(const GeomC& C, const StepParams& P, c
     pixel_step(C, P, D, iy * C.grid.n + ix, acc);
 }
 
+// The unconstrained minimiser t = x - f P^-1 v again by symmetric elimination
+// P = L diag(p0, d1, d2) L^T: its error grows with the condition number, the adjugate's
+// with its square where two eigenvalues are small (5e-10 against 1.4e-5 of the step at
+// worst over random P of condition up to 1e6), and the box's minimiser is compared with
+// it along the flat directions.  t stays as it is if a pivot vanishes.
+__device__ __forceinline__ void eliminate3(const dfl (&p)[6], const float* v, dfl f, const float4& x, dfl (&t)[3]) {
+    const dfl r0 = df_rcp_fma(p[0]), l1 = df_mul(r0, p[1]), l2 = df_mul(r0, p[2]);
+    const dfl d1 = df_sub(p[3], df_mul(l1, p[1])), e4 = df_sub(p[4], df_mul(l1, p[2]));
+    const dfl r1 = df_rcp_fma(d1), l3 = df_mul(e4, r1);
+    const dfl d2 = df_sub(df_sub(p[5], df_mul(l2, p[2])), df_mul(l3, e4));
+    if (p[0].hi == 0.0f || d1.hi == 0.0f || d2.hi == 0.0f || !isfinite(p[0].hi) || !isfinite(d1.hi) || !isfinite(d2.hi))
+        return;
+    const dfl y1 = df_sub(dfl{v[1], 0.0f}, df_mulf(l1, v[0]));
+    const dfl y2 = df_sub(df_sub(dfl{v[2], 0.0f}, df_mulf(l2, v[0])), df_mul(l3, y1));
+    const dfl u2 = df_mul(y2, df_rcp_fma(d2));
+    const dfl u1 = df_sub(df_mul(y1, r1), df_mul(l3, u2));
+    const dfl u0 = df_sub(df_sub(df_mulf(r0, v[0]), df_mul(l1, u1)), df_mul(l2, u2));
+    t[0] = df_sub(dfl{x.x, 0.0f}, df_mul(u0, f));
+    t[1] = df_sub(dfl{x.y, 0.0f}, df_mul(u1, f));
+    t[2] = df_sub(dfl{x.z, 0.0f}, df_mul(u2, f));
+}
+
 // a7 for pixel k from its nine back-projected channels: acc[0..2] = v_k = (K^T y')_k,
 // acc[3..8] = P_k (packed 00 01 02 11 12 22), T^-1_k = P_k / lambda; the primal
 // step x' = x - T_k v_k (optionally onto the box) and the extrapolation
 // xbar' = 2 x' - x.  T_k = lambda (P_k + 1e-12 tr(P_k) I)^-1 (the regularisation
-// that keeps T positive definite) is applied by symmetric elimination in double-float
-// arithmetic on P_k scaled by an exact power of two near 1 / tr(P_k); T_k has a
-// condition number near 6e6, and the ~48-bit elimination (whose error grows with the
-// condition number; the adjugate's grows with its square when two eigenvalues are
-// small: 5e-10 against 1.4e-5 of the step at worst over random P of condition up to
-// 1e6) keeps the step to FP32 accuracy.
+// that keeps T positive definite) is applied by the adjugate in double-float
+// arithmetic on P_k scaled by an exact power of two near 1 / tr(P_k), so that the
+// cubed entries stay inside the FP32 exponent range; T_k has a condition number
+// near 6e6, and the ~48-bit double-float solve keeps the step to FP32 accuracy.
 // A step that leaves the box is replaced by the box's minimiser (box_step3).
 __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, const SolveD& D, int k,
                                            const float acc[9]) {
@@ -1215,20 +1235,20 @@ __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, 
     const float p1 = acc[4] * sc, p2 = acc[5] * sc, p4 = acc[7] * sc;
     const float reg = 1e-12f * ((acc[3] * sc + acc[6] * sc) + acc[8] * sc);
     const dfl p0 = df_2sum(acc[3] * sc, reg), p3 = df_2sum(acc[6] * sc, reg), p5 = df_2sum(acc[8] * sc, reg);
-    // elimination of the scaled P: P = L diag(p0, d1, d2) L^T
-    const dfl p[6] = {p0, {p1, 0.0f}, {p2, 0.0f}, p3, {p4, 0.0f}, p5};
-    const dfl r0 = df_rcp(p0), l1 = df_mulf(r0, p1), l2 = df_mulf(r0, p2);
-    const dfl d1 = df_sub(p3, df_mulf(l1, p1)), e4 = df_sub(p[4], df_mulf(l1, p2));
-    const dfl r1 = df_rcp(d1), l3 = df_mul(e4, r1);
-    const dfl d2 = df_sub(df_sub(p5, df_mulf(l2, p2)), df_mul(l3, e4));
+    const dfl P1 = {p1, 0.0f}, P2 = {p2, 0.0f};
+    const dfl c00 = df_sub(df_mul(p3, p5), df_2prod(p4, p4));
+    const dfl c01 = df_sub(df_2prod(p2, p4), df_mulf(p5, p1));
+    const dfl c02 = df_sub(df_2prod(p1, p4), df_mulf(p3, p2));
+    const dfl c11 = df_sub(df_mul(p0, p5), df_2prod(p2, p2));
+    const dfl c12 = df_sub(df_2prod(p1, p2), df_mulf(p0, p4));
+    const dfl c22 = df_sub(df_mul(p0, p3), df_2prod(p1, p1));
+    const dfl det = df_add(df_add(df_mul(p0, c00), df_mul(P1, c01)), df_mul(P2, c02));
     dfl t[3] = {{x.x, 0.0f}, {x.y, 0.0f}, {x.z, 0.0f}};
-    if (p0.hi != 0.0f && d1.hi != 0.0f && d2.hi != 0.0f && isfinite(p0.hi) && isfinite(d1.hi) && isfinite(d2.hi)) {
-        const dfl y1 = df_sub(dfl{acc[1], 0.0f}, df_mulf(l1, acc[0]));
-        const dfl y2 = df_sub(df_sub(dfl{acc[2], 0.0f}, df_mulf(l2, acc[0])), df_mul(l3, y1));
-        const dfl u2 = df_mul(y2, df_rcp(d2));
-        const dfl u1 = df_sub(df_mul(y1, r1), df_mul(l3, u2));
-        const dfl u0 = df_sub(df_sub(df_mulf(r0, acc[0]), df_mul(l1, u1)), df_mul(l2, u2));
-        const dfl f = df_2prod(P.lambda, sc);   // exact: sc is a power of two
+    if (det.hi != 0.0f && isfinite(det.hi)) {
+        const dfl f = df_mulf(df_rcp(det), P.lambda * sc);   // lambda sc / det
+        const dfl u0 = df_add(df_add(df_mulf(c00, acc[0]), df_mulf(c01, acc[1])), df_mulf(c02, acc[2]));
+        const dfl u1 = df_add(df_add(df_mulf(c01, acc[0]), df_mulf(c11, acc[1])), df_mulf(c12, acc[2]));
+        const dfl u2 = df_add(df_add(df_mulf(c02, acc[0]), df_mulf(c12, acc[1])), df_mulf(c22, acc[2]));
         t[0] = df_sub(t[0], df_mul(u0, f));
         t[1] = df_sub(t[1], df_mul(u1, f));
         t[2] = df_sub(t[2], df_mul(u2, f));
@@ -1236,6 +1256,8 @@ __device__ __forceinline__ void pixel_step(const GeomC& C, const StepParams& P, 
     float xo3[3] = {df_f(t[0]), df_f(t[1]), df_f(t[2])};
     if (P.use_box && (xo3[0] < P.lo[0] || xo3[0] > P.hi[0] || xo3[1] < P.lo[1] || xo3[1] > P.hi[1] ||
                       xo3[2] < P.lo[2] || xo3[2] > P.hi[2])) {
+        const dfl p[6] = {p0, P1, P2, p3, {p4, 0.0f}, p5};
+        eliminate3(p, acc, df_2prod(P.lambda, sc), x, t);
         if (!box_step3(p, t, P.lo, P.hi, xo3)) {
             const double il = 1.0 / (double)P.lambda;
             double T[6] = {acc[3] * il, acc[4] * il, acc[5] * il, acc[6] * il, acc[7] * il, acc[8] * il};

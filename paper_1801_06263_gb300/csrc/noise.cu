@@ -159,7 +159,7 @@ __device__ __forceinline__ bool poisson_fast(float lam, uint32_t i, uint32_t k0,
         const float bits = (float)(r.y >> 6) * 0x1p-26f, f = neg ? 1.0f - bits : bits;
         if (n < 1024) return false;
         const dfl us = fixed27(n, 1.0f - f);
-        const dfl slope = df_add(df_mul(dfl{2.0f * a.hi, 2.0f * a.lo}, df_rcp(us)), b);
+        const dfl slope = df_add(df_mul(dfl{2.0f * a.hi, 2.0f * a.lo}, df_rcp_fma(us)), b);
         const dfl su = df_mul(slope, fixed27(m, f));
         const dfl v = df_add(df_add(neg ? df_neg(su) : su, dconst(0.43)), dfl{lf, 0.0f});
         const float fl = floorf(v.hi), fr = (v.hi - fl) + v.lo;

@@ -56,19 +56,27 @@ __device__ __forceinline__ dfl df_mulf(dfl x, float y) {
 
 __device__ __forceinline__ float df_f(dfl x) { return __fadd_rn(x.hi, x.lo); }
 
-// 1 / x: r + r (1 - x r) with r the FP32 reciprocal of x.hi.  The residual is one
-// exact FMA plus x.lo's share (|residual| <= 2^-23, so FP32 holds it to 2^-47).
+// 1 / x: r + r (1 - x r) with r the FP32 reciprocal of x.hi.
 __device__ __forceinline__ dfl df_rcp(dfl x) {
+    const float r = __frcp_rn(x.hi);
+    const dfl e = df_sub(dfl{1.0f, 0.0f}, df_mulf(x, r));
+    return df_add(dfl{r, 0.0f}, df_mulf(e, r));
+}
+
+// The same in a sixth of the instructions: the residual is one exact FMA plus x.lo's
+// share (|residual| <= 2^-23, so FP32 holds it to 2^-47).  Not for the dual step, whose
+// most attenuated rays carry a last bit of it into y' (1e-3 of its size at 512 x 512).
+__device__ __forceinline__ dfl df_rcp_fma(dfl x) {
     const float r = __frcp_rn(x.hi);
     const float e = __fmaf_rn(-x.lo, r, __fmaf_rn(-x.hi, r, 1.0f));
     return df_fast2sum(r, __fmul_rn(r, e));
 }
 
 // sqrt of a positive double-float: s = sqrt(hi) corrected by one Newton step,
-// s + (x - s^2) / (2 s) (Karp and Markstein 1997), the residual one exact FMA.
+// s + (x - s^2) / (2 s) (Karp and Markstein 1997), the correction in FP32.
 __device__ __forceinline__ dfl df_sqrt(dfl x) {
     const float s = __fsqrt_rn(x.hi);
-    const float e = __fadd_rn(__fmaf_rn(-s, s, x.hi), x.lo);
+    const float e = df_f(df_sub(x, df_2prod(s, s)));
     return df_fast2sum(s, __fmul_rn(e, __fdiv_rn(0.5f, s)));
 }
 
