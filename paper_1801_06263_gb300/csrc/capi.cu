@@ -51,7 +51,7 @@ void free_ctx(osscir_ctx* h) {
         if (e) cudaEventDestroy(e);
     if (h->fork) cudaEventDestroy(h->fork);
     if (h->join) cudaEventDestroy(h->join);
-    void* ptrs[] = {h->rec,     h->r64,    h->views,     h->chord,    h->exc_off,    h->exc_ent,  h->s4,
+    void* ptrs[] = {h->scratch, h->rec,     h->r64,    h->views,     h->chord,    h->exc_off,    h->exc_ent,  h->s4,
                     h->N4,      h->mu,     h->mu_in,     h->g,        h->c,          h->y,        h->x,
                     h->xbar,    h->xo,     h->dtpl_part, h->dtpl_out, h->bad_counts, h->model,    h->fwd_unit,
                     h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit, h->bp_w,
@@ -292,19 +292,16 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     CK(cudaEventCreateWithFlags(&h->join, cudaEventDisableTiming));
     cudaStream_t st = h->cap_stream;
 
-    // spectral tables: s reordered to [nE][n_bins] window vectors (4 F4 floats, zero padded)
-    // so consecutive rays read consecutive entries
+    // spectral tables, laid out on the device; the exception offsets' prefix sum goes first
+    const size_t n_scan = 2 * (1 + scan_scratch((size_t)L));   // in floats
     {
-        const int S = 4 * F4;
-        std::vector<float> s4((size_t)nE * g->n_bins * S, 0.0f), N4((size_t)g->n_bins * S, 0.0f);
-        for (int b = 0; b < g->n_bins; ++b)
-            for (int i = 0; i < nE; ++i)
-                for (int w = 0; w < W; ++w)
-                    s4[((size_t)i * g->n_bins + b) * S + w] = sp->s[((size_t)b * nE + i) * W + w];
-        for (int b = 0; b < g->n_bins; ++b)
-            for (int w = 0; w < W; ++w) N4[(size_t)b * S + w] = sp->N[(size_t)b * W + w];
-        CK(cudaMemcpy(h->s4, s4.data(), s4.size() * sizeof(float), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(h->N4, N4.data(), N4.size() * sizeof(float), cudaMemcpyHostToDevice));
+        const size_t ns = (size_t)nE * g->n_bins * W, nN = (size_t)g->n_bins * W;
+        CK(dalloc(&h->scratch, n_scan + ns + nN));
+        float* s_in = h->scratch + n_scan;
+        CK(cudaMemcpyAsync(s_in, sp->s, ns * sizeof(float), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(s_in + ns, sp->N, nN * sizeof(float), cudaMemcpyHostToDevice, st));
+        CK(launch_spectra(s_in, s_in + ns, g->n_bins, nE, W, 4 * F4, reinterpret_cast<float*>(h->s4),
+                          reinterpret_cast<float*>(h->N4), st));
         if (h->basis) {
             std::vector<double> mu_t;
             if (!mu_pc_basis(mu, nE, h->Mb, mu_t)) return OSSCIR_E_INVALID;
@@ -317,20 +314,13 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     }
     // per-ray records, then the footprint pairs decided in FP64
     CK(launch_ray_setup(G, r_img, h->rec, h->r64, h->views, st));
-    CK(launch_exc_pass(C, G, h->rec, h->r64, h->exc_off, nullptr, nullptr, st));
-    std::vector<int> cnt(L + 1, 0);
-    CK(cudaMemcpyAsync(cnt.data(), h->exc_off, sizeof(int) * L, cudaMemcpyDeviceToHost, st));
+    CK(launch_exc_pass(C, G, h->rec, h->r64, reinterpret_cast<uint32_t*>(h->exc_off), nullptr, nullptr, st));
+    unsigned long long run = 0, *run_d = reinterpret_cast<unsigned long long*>(h->scratch);
+    CK(launch_scan(reinterpret_cast<uint32_t*>(h->exc_off) + 1, (size_t)L, run_d, st));
+    CK(cudaMemcpyAsync(&run, run_d, sizeof run, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    long long run = 0;
-    for (int l = 0; l < L; ++l) {
-        const int c0 = cnt[l];
-        cnt[l] = (int)run;
-        run += c0;
-    }
-    if (run > (1LL << 31) - 1) return OSSCIR_E_NOMEM;
-    cnt[L] = (int)run;
+    if (run > (1ULL << 31) - 1) return OSSCIR_E_NOMEM;
     h->exc_n = (int)run;
-    CK(cudaMemcpyAsync(h->exc_off, cnt.data(), sizeof(int) * (L + 1), cudaMemcpyHostToDevice, st));
     CK(dalloc(&h->exc_ent, run));
     CK(launch_exc_pass(C, G, h->rec, h->r64, nullptr, h->exc_off, h->exc_ent, st));
     CK(launch_chord(C, h->exc(), h->rec, h->chord, st));
@@ -341,6 +331,9 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     CK(cudaMemsetAsync(h->dtpl_out, 0, sizeof(double) * 2, st));
     CK(cudaMemsetAsync(h->bad_counts, 0, 2 * sizeof(int), st));
     CK(cudaStreamSynchronize(st));
+    cudaFree(h->scratch);
+    h->scratch = nullptr;
+    h->bytes -= sizeof(float) * (n_scan + ((size_t)nE + 1) * g->n_bins * W);
     return OSSCIR_OK;
 }
 
@@ -394,33 +387,39 @@ osscir_status build_tables(osscir_ctx* h) {
     // forward: per-ray counts and per-warp rows, then the pairs
     CKT(dalloc(&h->fwd_cnt, (size_t)h->L));
     CKT(dalloc(&h->fwd_unit, n_fw + 1));
+    const int n_t = bt_tiles(C.grid.n), per = (C.n_views + G - 1) / G;
     struct {
-        unsigned long long total, fwd_total;
         int most[kBTSizes], wide, bad;   // bad: a pixel step outside 16 bits
+        unsigned long long total[2];     // forward and back-projection units
     } stat{};
+    // its copy on the device, the last total followed by the prefix sums' scratch
     char* stat_d = nullptr;
-    CKT(dalloc(&stat_d, sizeof stat));
+    const size_t stat_bytes =
+        sizeof stat + sizeof(unsigned long long) * scan_scratch(std::max(n_fw, (size_t)n_t * (C.n_views + 8) * kBTWarps));
+    CKT(dalloc(&stat_d, stat_bytes));
     auto dev = [&](auto* field) {   // where the field lies on the device
         return reinterpret_cast<decltype(field)>(stat_d + (reinterpret_cast<char*>(field) - reinterpret_cast<char*>(&stat)));
     };
+    unsigned long long* run_d = dev(&stat.total[1]);
     auto read_stat = [&]() {
         cudaError_t r = cudaMemcpyAsync(&stat, stat_d, sizeof stat, cudaMemcpyDeviceToHost, st);
         return r != cudaSuccess ? r : cudaStreamSynchronize(st);
     };
     cudaError_t e = cudaMemsetAsync(stat_d, 0, sizeof stat, st);
     if (e == cudaSuccess) e = launch_fp_fwd_count(C, h->exc(), h->rec, h->fwd_cnt, h->fwd_unit, st);
-    if (e == cudaSuccess) e = launch_scan(h->fwd_unit + 1, n_fw, dev(&stat.fwd_total), st);
+    if (e == cudaSuccess) e = launch_scan(h->fwd_unit + 1, n_fw, run_d, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(dev(&stat.total[0]), run_d, sizeof *run_d, cudaMemcpyDeviceToDevice, st);
     // back-projection (blocked): per tile and view the bins that can meet it; the chunk
     // size (views per staged chunk) whose two stage buffers fit; the units of each
     // (block, warp, chunk) and their prefix sum; then the entries
-    const int n_t = bt_tiles(C.grid.n), per = (C.n_views + G - 1) / G;
     if (e == cudaSuccess) e = dalloc(&h->bp_span, (size_t)n_t * C.n_views);
     if (e == cudaSuccess) e = launch_fpb_span(C, h->views, G, h->bp_span, dev(&stat.most[0]), st);
     if (e == cudaSuccess) e = read_stat();
     // forward: the pairs; one more unit than the table has (it is loaded ahead)
-    if (e == cudaSuccess && stat.fwd_total > 0xffffffffull) e = cudaErrorMemoryAllocation;
-    if (e == cudaSuccess) e = dalloc(&h->fwd_w, ((size_t)stat.fwd_total + 1) * 128);
-    if (e == cudaSuccess) e = dalloc(&h->fwd_d, ((size_t)stat.fwd_total + 1) * 128);
+    if (e == cudaSuccess && stat.total[0] > 0xffffffffull) e = cudaErrorMemoryAllocation;
+    if (e == cudaSuccess) e = dalloc(&h->fwd_w, ((size_t)stat.total[0] + 1) * 128);
+    if (e == cudaSuccess) e = dalloc(&h->fwd_d, ((size_t)stat.total[0] + 1) * 128);
     if (e == cudaSuccess) e = dalloc(&h->fwd_k0, (size_t)h->L);
     if (e == cudaSuccess)
         e = launch_fp_fwd_fill(C, h->exc(), h->rec, h->fwd_unit, h->fwd_w, h->fwd_d, h->fwd_k0, dev(&stat.bad), st);
@@ -435,19 +434,19 @@ osscir_status build_tables(osscir_ctx* h) {
         e = dalloc(&h->bp_unit, n_u + 1);
         if (e == cudaSuccess)
             e = launch_fpb_count(C, h->exc(), h->rec, h->views, h->fp(), h->bp_unit, dev(&stat.wide), st);
-        if (e == cudaSuccess) e = launch_scan(h->bp_unit + 1, n_u, dev(&stat.total), st);
+        if (e == cudaSuccess) e = launch_scan(h->bp_unit + 1, n_u, run_d, st);
         if (e == cudaSuccess) e = read_stat();
-        if (e == cudaSuccess && stat.total > 0xffffffffull) e = cudaErrorMemoryAllocation;
+        if (e == cudaSuccess && stat.total[1] > 0xffffffffull) e = cudaErrorMemoryAllocation;
         h->bp_wide = stat.wide;
         if (e == cudaSuccess) e = dalloc(&h->bp_part, (size_t)G * 9 * h->P);
-        if (e == cudaSuccess) e = dalloc(&h->bp_slot, ((size_t)stat.total + 1) * (stat.wide ? 64 : 32));
-        if (e == cudaSuccess) e = dalloc(&h->bp_w, ((size_t)stat.total + 1) * 64);   // one more unit: it is loaded ahead
+        if (e == cudaSuccess) e = dalloc(&h->bp_slot, ((size_t)stat.total[1] + 1) * (stat.wide ? 64 : 32));
+        if (e == cudaSuccess) e = dalloc(&h->bp_w, ((size_t)stat.total[1] + 1) * 64);   // one more unit: it is loaded ahead
         if (e == cudaSuccess) e = launch_fpb_fill(C, h->exc(), h->rec, h->views, h->fp(), h->bp_w, h->bp_slot, st);
     }
     if (e == cudaSuccess) e = read_stat();
     if (e == cudaSuccess && stat.bad) e = cudaErrorMemoryAllocation;
     cudaFree(stat_d);
-    h->bytes -= sizeof stat;
+    h->bytes -= stat_bytes;
     CKT(e);
     CKT(cudaStreamSynchronize(st));
 #undef CKT

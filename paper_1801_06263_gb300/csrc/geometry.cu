@@ -83,28 +83,66 @@ __global__ void k_view_setup(GeomD G, ViewF* views) {
     views[v] = ViewF{(float)cos(th), (float)sin(th)};
 }
 
-// Ambiguous candidates (FP32 chord within its error bound of zero) decided in
-// FP64; count == nullptr selects the fill pass.
-__global__ void k_exc_pass(GeomC C, GeomD G, const RayRec* rec, const Ray64* r64, int* count,
-                           const int* off, int2* ent, int L) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+// Ambiguous candidates (FP32 chord within its error bound of zero) decided in FP64;
+// count != nullptr counts them per ray (count[0] = 0, ray l's at count[1 + l]), else
+// they are filled in at ent[off[l] ..].  A warp per ray, its slabs along the dominant
+// axis over the lanes: a ray (nearly) parallel to an axis has all its pixels decided in
+// FP64, and with a thread per ray those few rays, 512 FP64 chords in a row, took the
+// pass 2970 us at 256 x 256 (667 us this way, and the second pass skips the many rays
+// without an entry).  Lane order is slab order, so the keys come out sorted.
+__global__ void __launch_bounds__(128) k_exc_pass(GeomC C, GeomD G, const RayRec* rec, const Ray64* r64, uint32_t* count,
+                                                  const int* off, int2* ent, int L) {
+    const int l = (int)(blockIdx.x * 4 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
     if (l >= L) return;
     const float4 r0 = rec[l].r0;
     const float ex = rec[l].r1.x, ey = rec[l].r1.y;
-    const Ray64 R = r64[l];
-    int cnt = 0;
-    const int base = count ? 0 : off[l];
     const bool rows = ray_rows(r0);
-    // ray_chords enumerates (major, minor) in increasing order, so the keys come out sorted
-    ray_chords(r0, ex, ey, C.grid, C.margin_mm, [&](int ix, int iy, float w, float eb) {
-        if (w > eb || w < -eb) return;
-        const double c64 = chord64(R, G, ix, iy);
-        if (c64 > G.thr) {
-            if (!count) ent[base + cnt] = make_int2(exc_key(rows, C.grid.n, ix, iy), __float_as_int((float)c64));
-            ++cnt;
+    int jlo, jhi;
+    int cnt = 0;
+    if (ray_slabs(r0, C.grid, C.margin_mm, jlo, jhi)) {
+        const int base = count ? 0 : off[l];
+        if (!count && off[l + 1] == base) return;   // most rays have none
+        for (int j0 = jlo; j0 <= jhi; j0 += 32) {
+            int2 found[3];
+            int n = 0;
+            const int j = j0 + lane;
+            if (j <= jhi) {
+                const auto visit = [&](int ix, int iy, float w, float eb) {
+                    if (w > eb || w < -eb) return;
+                    const double c64 = chord64(r64[l], G, ix, iy);
+                    if (c64 > G.thr) {
+                        const int2 e = make_int2(exc_key(rows, C.grid.n, ix, iy), __float_as_int((float)c64));
+                        if (n == 0) found[0] = e;
+                        else if (n == 1) found[1] = e;
+                        else found[2] = e;
+                        ++n;
+                    }
+                };
+                if (rows) slab_chords<true>(r0, ex, ey, C.grid, C.margin_mm, j, visit);
+                else slab_chords<false>(r0, ex, ey, C.grid, C.margin_mm, j, visit);
+            }
+            if (!__any_sync(0xffffffffu, n > 0)) continue;
+            int before = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, before, o);
+                if (lane >= o) before += v;
+            }
+            const int all = __shfl_sync(0xffffffffu, before, 31);
+            before -= n;
+            if (!count) {
+                int2* to = ent + base + cnt + before;
+                if (n > 0) to[0] = found[0];
+                if (n > 1) to[1] = found[1];
+                if (n > 2) to[2] = found[2];
+            }
+            cnt += all;
         }
-    });
-    if (count) count[l] = cnt;
+    }
+    if (count && lane == 0) {
+        count[1 + l] = (uint32_t)cnt;
+        if (l == 0) count[0] = 0;
+    }
 }
 
 // (X 1)_l = sum_k X_{l,k}: the chord of each ray through the image.
@@ -175,10 +213,31 @@ cudaError_t launch_ray_setup(const GeomD& G, double r_img, RayRec* rec, Ray64* r
     return cudaGetLastError();
 }
 
-cudaError_t launch_exc_pass(const GeomC& C, const GeomD& G, const RayRec* rec, const Ray64* r64, int* count,
+cudaError_t launch_exc_pass(const GeomC& C, const GeomD& G, const RayRec* rec, const Ray64* r64, uint32_t* count,
                             const int* off, int2* ent, cudaStream_t st) {
     const int L = G.n_views * G.n_bins;
-    k_exc_pass<<<blocks(L, 128), 128, 0, st>>>(C, G, rec, r64, count, off, ent, L);
+    k_exc_pass<<<blocks(L, 4), 128, 0, st>>>(C, G, rec, r64, count, off, ent, L);
+    return cudaGetLastError();
+}
+
+// s4 [nE][n_bins] and N4 [n_bins] window vectors from the caller's s [n_bins][nE][W] and
+// N [n_bins][W], zero padded: consecutive rays read consecutive entries.
+__global__ void k_spectra(const float* __restrict__ s, const float* __restrict__ N, int n_bins, int nE, int W, int S,
+                          float* s4, float* N4) {
+    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (i < (size_t)nE * n_bins * S) {
+        const int w = (int)(i % S), b = (int)(i / S % n_bins), e = (int)(i / S / n_bins);
+        s4[i] = w < W ? s[((size_t)b * nE + e) * W + w] : 0.0f;
+    }
+    if (i < (size_t)n_bins * S) {
+        const int w = (int)(i % S), b = (int)(i / S);
+        N4[i] = w < W ? N[(size_t)b * W + w] : 0.0f;
+    }
+}
+
+cudaError_t launch_spectra(const float* s, const float* N, int n_bins, int nE, int W, int S, float* s4, float* N4,
+                           cudaStream_t st) {
+    k_spectra<<<(unsigned)(((size_t)nE * n_bins * S + 255) / 256), 256, 0, st>>>(s, N, n_bins, nE, W, S, s4, N4);
     return cudaGetLastError();
 }
 

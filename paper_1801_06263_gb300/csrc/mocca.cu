@@ -1366,10 +1366,20 @@ __global__ void __launch_bounds__(kFwdThreads) k_fp_fwd_fill(GeomC C, ExcTable E
     const float4 r0 = rec[l].r0, r1 = rec[l].r1;
     int j = 0, prev = -1;
     bool col = false;
+    float w0 = 0.f, w1 = 0.f, w2 = 0.f;   // the first three pairs of the unit under way
+    uint32_t d01 = 0, d2 = 0;
     auto put = [&](int d, float w) {
-        const size_t at = ((q0 + (j >> 2)) * 32 + lane) * 4 + (j & 3);
-        fwd_w[at] = w;
-        fwd_d[at] = (int16_t)d;
+        const uint32_t dd = (uint32_t)d & 0xffffu;
+        switch (j & 3) {
+            case 0: w0 = w, d01 = dd; break;
+            case 1: w1 = w, d01 |= dd << 16; break;
+            case 2: w2 = w, d2 = dd; break;
+            default: {
+                const size_t at = (q0 + (j >> 2)) * 32 + lane;
+                reinterpret_cast<float4*>(fwd_w)[at] = make_float4(w0, w1, w2, w);
+                reinterpret_cast<uint2*>(fwd_d)[at] = make_uint2(d01, d2 | dd << 16);
+            }
+        }
         ++j;
     };
     ray_pixels(C, E, r0, r1.x, r1.y, l, [&](int kr, float w) {
@@ -1619,10 +1629,13 @@ __global__ void __launch_bounds__(kBTThreads) k_fpb_count(GeomC C, ExcTable E, c
     if (far) *wide = 1;
 }
 
-// Table pass 2: every row of every unit.
+// Table pass 2: every row of every unit.  A thread's entries of a view wait in shared
+// memory for the warp's row count (up to kBTKeep of them; more are found again).
+constexpr int kBTKeep = 8;
 __global__ void __launch_bounds__(kBTThreads) k_fpb_fill(GeomC C, ExcTable E, const RayRec* rec,
                                                          const ViewF* views, FpTables T, float4* bp_w,
                                                          uint32_t* bp_slot) {
+    __shared__ float2 keep[kBTKeep][kBTThreads];
     const int G = T.bp_groups, nch = T.bp_nch, b = blockIdx.x, t = b / G, g = b % G, tid = threadIdx.x, lane = tid & 31;
     int ix, iy;
     bt_pixel(C.grid.n, t, tid, ix, iy);
@@ -1646,11 +1659,18 @@ __global__ void __launch_bounds__(kBTThreads) k_fpb_fill(GeomC C, ExcTable E, co
         };
         for (int u = u0; u < u1; ++u) {
             int n = 0, first = 0;
-            if (valid) n = pair_entries(C, E, rec, views[u], u, ix, iy, first, [](int, float, float) {});
+            if (valid)
+                n = pair_entries(C, E, rec, views[u], u, ix, iy, first, [&](int j, float w0, float w1) {
+                    if (j < kBTKeep) keep[j][tid] = make_float2(w0, w1);
+                });
             const int K = __reduce_max_sync(0xffffffffu, n);
             if (n > 0) {
                 const int s0 = off[u - u0] + first - tlo[u - u0];
-                pair_entries(C, E, rec, views[u], u, ix, iy, first, [&](int j, float w0, float w1) { put(s0 + j, w0, w1); });
+                if (n <= kBTKeep)
+                    for (int j = 0; j < n; ++j) put(s0 + j, keep[j][tid].x, keep[j][tid].y);
+                else
+                    pair_entries(C, E, rec, views[u], u, ix, iy, first,
+                                 [&](int j, float w0, float w1) { put(s0 + j, w0, w1); });
                 slot = s0 + n - 1;
             }
             for (int j = n; j < K; ++j) put(slot, 0.0f, 0.0f);
@@ -1916,46 +1936,69 @@ __global__ void __launch_bounds__(kFinishThreads) k_fpb_finish(GeomC C, StepPara
     }
 }
 
-// In-place inclusive prefix sum by one block: each thread takes kScanEach
-// consecutive values of a tile, the tiles follow one another.
-constexpr int kScanThreads = 1024, kScanEach = 16;
-__global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* v, size_t n, unsigned long long* total) {
-    __shared__ unsigned long long warp_sum[kScanThreads / 32];
+// In-place inclusive prefix sum in three passes: the sums of tiles of kScanTile values,
+// their own (exclusive) prefix sum by one block, and the values from both.
+constexpr int kScanThreads = 1024, kScanTile = 4 * kScanThreads;
+
+// Inclusive prefix sum of x over the block's threads; *all gets the block's sum.
+template <class T>
+__device__ __forceinline__ T block_scan(T x, T* all) {
+    __shared__ T warp_sum[kScanThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long carry = 0;
-    for (size_t base = 0; base < n; base += (size_t)kScanThreads * kScanEach) {
-        const size_t i0 = base + (size_t)threadIdx.x * kScanEach;
-        uint32_t x[kScanEach];
-        unsigned long long own = 0;
 #pragma unroll
-        for (int j = 0; j < kScanEach; ++j) {
-            x[j] = i0 + j < n ? v[i0 + j] : 0u;
-            own += x[j];
-        }
-        unsigned long long inc = own;
+    for (int o = 1; o < 32; o <<= 1) {
+        const T u = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += u;
+    }
+    __syncthreads();   // a previous call's sums have been read
+    if (lane == 31) warp_sum[wid] = x;
+    __syncthreads();
+    T w = warp_sum[lane];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long u = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += u;
-        }
-        if (lane == 31) warp_sum[wid] = inc;
-        __syncthreads();
-        unsigned long long before = carry, all = 0;
-        for (int w = 0; w < kScanThreads / 32; ++w) {
-            const unsigned long long u = warp_sum[w];
-            before += w < wid ? u : 0ull;
-            all += u;
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const T u = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += u;
+    }
+    *all = __shfl_sync(0xffffffffu, w, 31);
+    const T before = __shfl_sync(0xffffffffu, w, max(wid - 1, 0));
+    return wid > 0 ? x + before : x;
+}
+
+__device__ __forceinline__ void scan_load(const uint32_t* v, size_t n, size_t i0, uint32_t (&x)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = i0 + j < n ? v[i0 + j] : 0u;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const uint32_t* v, size_t n, unsigned long long* sums) {
+    uint32_t x[4];
+    scan_load(v, n, (size_t)blockIdx.x * kScanTile + 4 * threadIdx.x, x);
+    unsigned long long all;
+    block_scan((unsigned long long)x[0] + x[1] + x[2] + x[3], &all);
+    if (threadIdx.x == 0) sums[blockIdx.x] = all;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_top(unsigned long long* sums, size_t n, unsigned long long* total) {
+    unsigned long long carry = 0, all;
+    for (size_t i0 = 0; i0 < n; i0 += kScanThreads) {
+        const size_t i = i0 + threadIdx.x;
+        const unsigned long long own = i < n ? sums[i] : 0ull, inc = block_scan(own, &all);
+        if (i < n) sums[i] = carry + inc - own;
         carry += all;
-        unsigned long long run = before + inc - own;
-#pragma unroll
-        for (int j = 0; j < kScanEach; ++j) {
-            run += x[j];
-            if (i0 + j < n) v[i0 + j] = (uint32_t)run;
-        }
-        __syncthreads();
     }
     if (threadIdx.x == 0) *total = carry;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(uint32_t* v, size_t n, const unsigned long long* sums) {
+    uint32_t x[4];
+    const size_t i0 = (size_t)blockIdx.x * kScanTile + 4 * threadIdx.x;
+    scan_load(v, n, i0, x);
+    const uint32_t own = x[0] + x[1] + x[2] + x[3];
+    uint32_t all, run = (uint32_t)sums[blockIdx.x] + block_scan(own, &all) - own;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        run += x[j];
+        if (i0 + j < n) v[i0 + j] = run;
+    }
 }
 
 constexpr int kReduceThreads = 1024;
@@ -2222,9 +2265,14 @@ cudaError_t launch_fpb_fill(const GeomC& C, const ExcTable& E, const RayRec* rec
 }
 
 cudaError_t launch_scan(uint32_t* v, size_t n, unsigned long long* total, cudaStream_t st) {
-    k_scan<<<1, kScanThreads, 0, st>>>(v, n, total);
+    const size_t tiles = scan_scratch(n);
+    k_scan_sums<<<(unsigned)tiles, kScanThreads, 0, st>>>(v, n, total + 1);
+    k_scan_top<<<1, kScanThreads, 0, st>>>(total + 1, tiles, total);
+    k_scan_apply<<<(unsigned)tiles, kScanThreads, 0, st>>>(v, n, total + 1);
     return cudaGetLastError();
 }
+
+size_t scan_scratch(size_t n) { return (n + kScanTile - 1) / kScanTile; }
 
 cudaError_t launch_mocca_apply(const GeomC& C, const StepParams& P, const SolveD& D, const float* chan,
                                cudaStream_t st) {

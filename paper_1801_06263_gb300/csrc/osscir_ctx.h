@@ -24,6 +24,7 @@ struct osscir_ctx {
     int* exc_off = nullptr;
     int2* exc_ent = nullptr;
     int exc_n = 0;
+    float* scratch = nullptr;   // held while the context is created only
     // spectral tables
     float4* s4 = nullptr;   // [nE][n_bins] window vectors
     float4* N4 = nullptr;   // [n_bins] window vectors

@@ -183,67 +183,59 @@ __device__ __forceinline__ int sat_floor(float v) {
     return static_cast<int>(floorf(fminf(fmaxf(v, -1.0e9f), 1.0e9f)));
 }
 
-// Candidate enumeration of a ray's pixels with their chords: slabs along the
-// dominant axis (ROWS: y), within each slab the minor-axis cells the ray can
-// touch (with a margin that exceeds the FP32 error of the crossing points).
-// Every plane parameter is computed once and shared by the neighbouring
-// cells; the chord and bound equal chord32's bit for bit.  Calls
-// visit(ix, iy, w, eb) for a superset of the footprint.
-template <bool ROWS, class Visit>
-__device__ __forceinline__ void ray_chords_dir(const float4& r0, float ex, float ey, const GridF& G, float margin,
-                                               Visit&& visit) {
-    const float bM = ROWS ? r0.y : r0.x, bm = ROWS ? r0.x : r0.y;
-    const float iM = ROWS ? r0.w : r0.z, im = ROWS ? r0.z : r0.w;
+// The slabs [jlo, jhi] along a ray's dominant axis that can hold pixels of it; false
+// if there are none.
+__device__ __forceinline__ bool ray_slabs(const float4& r0, const GridF& G, float margin, int& jlo, int& jhi) {
+    const bool rows = ray_rows(r0);
+    const float bM = rows ? r0.y : r0.x, bm = rows ? r0.x : r0.y;
+    const float iM = rows ? r0.w : r0.z, im = rows ? r0.z : r0.w;
     const float slope = iM / im;   // d_minor / d_major, |slope| <= 1 (0 for axis-parallel rays)
     const float xlo = G.x0, xhi = grid_plane(G, G.n);
-    int jlo = 0, jhi = G.n - 1;
+    jlo = 0, jhi = G.n - 1;
     if (slope != 0.0f) {
         const float ya = bM + (xlo - margin - bm) / slope;
         const float yb = bM + (xhi + margin - bm) / slope;
         jlo = max(jlo, sat_floor((fminf(ya, yb) - G.x0) / G.h) - 1);
         jhi = min(jhi, sat_floor((fmaxf(ya, yb) - G.x0) / G.h) + 1);
-    } else if (bm < xlo - margin || bm > xhi + margin) {
-        return;
+        return jlo <= jhi;
     }
-    const float inv_h = 1.0f / G.h;
-    float pM0 = grid_plane(G, jlo);
-    float tM0 = t_plane(pM0, bM, iM);
-    for (int j = jlo; j <= jhi; ++j) {
-        const float pM1 = grid_plane(G, j + 1);
-        const float tM1 = t_plane(pM1, bM, iM);
-        const float ma = fmaf(slope, pM0 - bM, bm), mb = fmaf(slope, pM1 - bM, bm);
-        const int ilo = max(sat_floor((fminf(ma, mb) - margin - G.x0) * inv_h), 0);
-        const int ihi = min(sat_floor((fmaxf(ma, mb) + margin - G.x0) * inv_h), G.n - 1);
-        if (ilo <= ihi) {
-            float tm0 = t_plane(grid_plane(G, ilo), bm, im);
-            for (int i = ilo; i <= ihi; ++i) {
-                const float tm1 = t_plane(grid_plane(G, i + 1), bm, im);
-                float w, eb;
-                if (ROWS) {
-                    chord_from_planes(tm0, tm1, tM0, tM1, r0.z, r0.w, ex, ey, w, eb);
-                    visit(i, j, w, eb);
-                } else {
-                    chord_from_planes(tM0, tM1, tm0, tm1, r0.z, r0.w, ex, ey, w, eb);
-                    visit(j, i, w, eb);
-                }
-                tm0 = tm1;
-            }
-        }
-        pM0 = pM1;
-        tM0 = tM1;
-    }
+    return !(bm < xlo - margin || bm > xhi + margin);
 }
 
-template <class Visit>
-__device__ __forceinline__ void ray_chords(const float4& r0, float ex, float ey, const GridF& G, float margin,
-                                           Visit&& visit) {
-    // r0.zw = (1/dx, 1/dy): the ray is row-major (|dy| >= |dx|) iff |1/dy| <= |1/dx|
-    if (ray_rows(r0)) ray_chords_dir<true>(r0, ex, ey, G, margin, visit);
-    else ray_chords_dir<false>(r0, ex, ey, G, margin, visit);
+// The candidate pixels of a ray in slab j of its dominant axis (ROWS: y) with their
+// chords: the minor-axis cells the ray can touch, at most three (with a margin that
+// exceeds the FP32 error of the crossing points), in increasing order.  Chord and bound
+// equal chord32's bit for bit.  Calls visit(ix, iy, w, eb) for a superset of the slab's
+// footprint.
+template <bool ROWS, class Visit>
+__device__ __forceinline__ void slab_chords(const float4& r0, float ex, float ey, const GridF& G, float margin, int j,
+                                            Visit&& visit) {
+    const float bM = ROWS ? r0.y : r0.x, bm = ROWS ? r0.x : r0.y;
+    const float iM = ROWS ? r0.w : r0.z, im = ROWS ? r0.z : r0.w;
+    const float slope = iM / im, inv_h = 1.0f / G.h;
+    const float pM0 = grid_plane(G, j), pM1 = grid_plane(G, j + 1);
+    const float tM0 = t_plane(pM0, bM, iM), tM1 = t_plane(pM1, bM, iM);
+    const float ma = fmaf(slope, pM0 - bM, bm), mb = fmaf(slope, pM1 - bM, bm);
+    const int ilo = max(sat_floor((fminf(ma, mb) - margin - G.x0) * inv_h), 0);
+    const int ihi = min(sat_floor((fmaxf(ma, mb) + margin - G.x0) * inv_h), G.n - 1);
+    if (ilo > ihi) return;
+    float tm0 = t_plane(grid_plane(G, ilo), bm, im);
+    for (int i = ilo; i <= ihi; ++i) {
+        const float tm1 = t_plane(grid_plane(G, i + 1), bm, im);
+        float w, eb;
+        if (ROWS) {
+            chord_from_planes(tm0, tm1, tM0, tM1, r0.z, r0.w, ex, ey, w, eb);
+            visit(i, j, w, eb);
+        } else {
+            chord_from_planes(tM0, tM1, tm0, tm1, r0.z, r0.w, ex, ey, w, eb);
+            visit(j, i, w, eb);
+        }
+        tm0 = tm1;
+    }
 }
 
 // X_{l,k} for every pixel of ray l with a nonzero weight: visit(k, w).  The
-// same slab enumeration as ray_chords, written once in (major, minor)
+// same slab enumeration as slab_chords, written once in (major, minor)
 // coordinates: the membership test is symmetric under exchanging the x and y
 // roles (fminf, fmaxf and chord_bound commute with the exchange), so one code
 // path serves both orientations and both direction signs, and every weight

@@ -119,8 +119,10 @@ inline int bp_view_groups(int n_pixels, int n_views) {
 
 cudaError_t launch_ray_setup(const GeomD& G, double r_img, RayRec* rec, Ray64* r64, ViewF* views,
                              cudaStream_t st);
-cudaError_t launch_exc_pass(const GeomC& C, const GeomD& G, const RayRec* rec, const Ray64* r64, int* count,
+cudaError_t launch_exc_pass(const GeomC& C, const GeomD& G, const RayRec* rec, const Ray64* r64, uint32_t* count,
                             const int* off, int2* ent, cudaStream_t st);
+cudaError_t launch_spectra(const float* s, const float* N, int n_bins, int nE, int W, int S, float* s4, float* N4,
+                           cudaStream_t st);
 cudaError_t launch_chord(const GeomC& C, const ExcTable& E, const RayRec* rec, float* chord, cudaStream_t st);
 cudaError_t launch_footprint_rays(const GeomC& C, const ExcTable& E, const RayRec* rec, int l0, int n, int cap,
                                   int* cnt, int* pix, float* wt, cudaStream_t st);
@@ -173,7 +175,9 @@ cudaError_t launch_fpb_span(const GeomC& C, const ViewF* views, int G, uint32_t*
 // of the former makes bp_unit); *wide set if a slot step does not fit a signed byte.
 cudaError_t launch_fpb_count(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
                              const FpTables& T, uint32_t* unit, int* wide, cudaStream_t st);
-// In-place inclusive prefix sum of v[0 .. n) modulo 2^32 (one block); *total the 64-bit sum.
+// In-place inclusive prefix sum of v[0 .. n) modulo 2^32; total[0] the 64-bit sum,
+// total[1 .. scan_scratch(n)] scratch.
+size_t scan_scratch(size_t n);
 cudaError_t launch_scan(uint32_t* v, size_t n, unsigned long long* total, cudaStream_t st);
 cudaError_t launch_fpb_fill(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
                             const FpTables& T, float4* bp_w, uint32_t* bp_slot, cudaStream_t st);
