@@ -671,8 +671,12 @@ __global__ void __launch_bounds__(kFwdThreads, 8) k_mocca_proj(GeomC C, ExcTable
 }
 
 // a2-a5 and the per-ray half of a8: spectral model, curvature, dual step.
-// Returns the ray's D_TPL terms; sm holds the block's mu table (load_mu_smem).
-template <bool KEEP, int W>
+// Returns the ray's D_TPL terms; sm holds the block's mu table (load_mu_smem).  CURV: with
+// the curvature sums U, which model 0 (the clipped Hessian) uses; without, the others save
+// their 28 of the 48 FP32 operations an energy (five windows, model 3, 256 x 256: the
+// kernel 114 -> 95 us).
+// EU: energies whose table loads are in flight together.
+template <bool KEEP, int W, bool CURV, int EU>
 __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P,
                                            const SolveD& D, const float* sm, int l) {
     static_assert(!KEEP || W == 4, "nested MOCCA keeps models of four windows");
@@ -701,7 +705,7 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
 #pragma unroll
             for (int w = 0; w < W; ++w) Pd[w] = 0.f;
             const int i1 = min(nE, i0 + kDFold);
-#pragma unroll 2   // two energies in flight: the s-table loads overlap
+#pragma unroll EU
             for (int i = i0; i < i1; ++i) {
                 const float4 qa = *reinterpret_cast<const float4*>(sm + kSmemStride * i);
                 const float4 qb = *reinterpret_cast<const float4*>(sm + kSmemStride * i + 4);
@@ -719,8 +723,9 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
                     An[w][0] = fmaf(a, qa.x, An[w][0]);
                     An[w][1] = fmaf(a, qa.y, An[w][1]);
                     An[w][2] = fmaf(a, qa.z, An[w][2]);
+                    if (CURV)
 #pragma unroll
-                    for (int k = 0; k < 6; ++k) U[w][k] = fmaf(c2, mm[k], U[w][k]);
+                        for (int k = 0; k < 6; ++k) U[w][k] = fmaf(c2, mm[k], U[w][k]);
                 }
             }
 #pragma unroll
@@ -786,7 +791,7 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
                 float t = qw[0] * U[0][k];
 #pragma unroll
                 for (int w = 1; w < W; ++w) t = fmaf(qw[w], U[w][k], t);
-                Bt[k] = P.model == 2 ? 0.0f : t;
+                Bt[k] = CURV && P.model != 2 ? t : 0.0f;
             }
             sigma_inv();
             ray_dual<KEEP, W>(al, sinv, cv, rw, Bt, y, yo, Bm);
@@ -837,14 +842,20 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
 // Resident blocks of 128 threads: five for four windows (96 registers, a few
 // spills; 0.137 ms at 256x256 against 0.144 ms with four and 0.160 ms with six),
 // four for five windows (128 registers; 0.136 ms against 0.152 ms with three).
-template <bool KEEP, int W>
-__global__ void __launch_bounds__(kFwdThreads, W == 4 ? 5 : 4) k_mocca_ray(GeomC C, RayRec* rec, SpecD S,
+// FEW: a grid of at most three blocks per SM has registers to spare and too few warps to
+// hide the spectral table's L2 latency, so eight energies' loads are in flight at once
+// (168 registers, no spills): 64 x 64 (128 blocks) 54 -> 42 us after an L2 flush, an
+// iteration 71 -> 66 us; 128 x 128 with 180 views (270 blocks) 62 -> 49 and 89 -> 84 us;
+// 630 blocks of 300 x 300 were 9 % slower with it.
+constexpr unsigned kRayFewBlocks = 3 * 152;
+template <bool KEEP, int W, bool CURV, bool FEW>
+__global__ void __launch_bounds__(kFwdThreads, FEW ? 3 : (W == 4 ? 5 : 4)) k_mocca_ray(GeomC C, RayRec* rec, SpecD S,
                                                                          StepParams P, SolveD D, int v0, int v1) {
     __shared__ float sm[kSmemStride * kMaxEnergies];
     load_mu_smem(S, sm);
     __syncthreads();
     const int l = ray_in_views(C, blockIdx.x, blockIdx.y, kFwdThreads / 32, v0, v1);
-    const double dsum = l >= 0 ? ray_step<KEEP, W>(C, rec, S, P, D, sm, l) : 0.0;
+    const double dsum = l >= 0 ? ray_step<KEEP, W, CURV, FEW ? 8 : 2>(C, rec, S, P, D, sm, l) : 0.0;
     warp_partial(C, blockIdx.x, v0 + warp_view(blockIdx.y, kFwdThreads / 32), dsum, D.dtpl_part, v1);
 }
 
@@ -2093,7 +2104,8 @@ __global__ void __launch_bounds__(kFwdThreads, 5) k_batch_ray(const SolveDesc* _
         const GeomC C = d.C;
         const int nbx = (C.n_bins + 31) >> 5, bx = w.y % nbx, by = w.y / nbx;
         const int l = ray_at(C, bx, by, kFwdThreads / 32);
-        const double dsum = l >= 0 ? ray_step<false, 4>(C, d.rec, d.S, d.P, d.D, sm, l) : 0.0;
+        // the one instance for every model: two in one kernel cost it 2 % (spills)
+        const double dsum = l >= 0 ? ray_step<false, 4, true, 2>(C, d.rec, d.S, d.P, d.D, sm, l) : 0.0;
         warp_partial(C, bx, warp_view(by, kFwdThreads / 32), dsum, d.D.dtpl_part);
     }
 }
@@ -2170,20 +2182,40 @@ cudaError_t launch_mocca_proj(const GeomC& C, const ExcTable& E, const RayRec* r
     return cudaGetLastError();
 }
 
+template <bool KEEP, int W, bool CURV>
+void launch_ray_grid(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P, const SolveD& D, int v0, int v1,
+                     cudaStream_t st) {
+    const dim3 grid = fwd_grid(C.n_bins, v1 - v0);
+    if (grid.x * grid.y <= kRayFewBlocks) k_mocca_ray<KEEP, W, CURV, true><<<grid, kFwdThreads, 0, st>>>(C, rec, S, P, D, v0, v1);
+    else k_mocca_ray<KEEP, W, CURV, false><<<grid, kFwdThreads, 0, st>>>(C, rec, S, P, D, v0, v1);
+}
+
+template <bool KEEP>
+void launch_ray(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P, const SolveD& D, int v0, int v1,
+                cudaStream_t st) {
+    const bool curv = P.model == 0;
+    if constexpr (!KEEP) {
+        if (S.n_windows == 5) {
+            if (curv) launch_ray_grid<false, 5, true>(C, rec, S, P, D, v0, v1, st);
+            else launch_ray_grid<false, 5, false>(C, rec, S, P, D, v0, v1, st);
+            return;
+        }
+    }
+    if (curv) launch_ray_grid<KEEP, 4, true>(C, rec, S, P, D, v0, v1, st);
+    else launch_ray_grid<KEEP, 4, false>(C, rec, S, P, D, v0, v1, st);
+}
+
 cudaError_t launch_mocca_ray(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P, const SolveD& D,
                              cudaStream_t st, int v0, int v1) {
     if (v1 < 0) v1 = C.n_views;
-    if (S.n_windows == 5)
-        k_mocca_ray<false, 5><<<fwd_grid(C.n_bins, v1 - v0), kFwdThreads, 0, st>>>(C, rec, S, P, D, v0, v1);
-    else
-        k_mocca_ray<false, 4><<<fwd_grid(C.n_bins, v1 - v0), kFwdThreads, 0, st>>>(C, rec, S, P, D, v0, v1);
+    launch_ray<false>(C, rec, S, P, D, v0, v1, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mocca_ray_keep(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P,
                                   const SolveD& D, cudaStream_t st) {
     if (S.n_windows != 4) return cudaErrorInvalidValue;   // nested MOCCA keeps four-window models
-    k_mocca_ray<true, 4><<<fwd_grid(C.n_bins, C.n_views), kFwdThreads, 0, st>>>(C, rec, S, P, D, 0, C.n_views);
+    launch_ray<true>(C, rec, S, P, D, 0, C.n_views, st);
     return cudaGetLastError();
 }
 
