@@ -137,17 +137,21 @@ cudaError_t launch_counts(const GeomC& C, const ExcTable& E, const RayRec* rec, 
                           float4* chat, const float4* c, double* dtpl_part, cudaStream_t st);
 // The ray-driven kernels over the views [v0, v1) (v1 < 0: all views); with
 // footprint tables T the projections stream them (same results bit for bit).
+// chained: launched as a programmatic dependent of the kernel before it in the stream,
+// which must be one of the iteration's with tables (no effect on a kernel without them).
 cudaError_t launch_mocca_proj(const GeomC& C, const ExcTable& E, const RayRec* rec, const SolveD& D,
-                              cudaStream_t st, int v0 = 0, int v1 = -1, const FpTables* T = nullptr);
+                              cudaStream_t st, int v0 = 0, int v1 = -1, const FpTables* T = nullptr, bool chained = false);
 cudaError_t launch_mocca_ray(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P, const SolveD& D,
-                             cudaStream_t st, int v0 = 0, int v1 = -1);
+                             cudaStream_t st, int v0 = 0, int v1 = -1, bool chained = false);
 // Outer iteration of nested MOCCA: the per-ray step that also keeps each ray's model in D.model.
 cudaError_t launch_mocca_ray_keep(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P,
-                                  const SolveD& D, cudaStream_t st);
+                                  const SolveD& D, cudaStream_t st, bool chained = false);
 // Inner iteration of nested MOCCA: the dual step on the kept models.
-cudaError_t launch_mocca_ray_inner(const GeomC& C, RayRec* rec, const SolveD& D, cudaStream_t st);
+cudaError_t launch_mocca_ray_inner(const GeomC& C, RayRec* rec, const SolveD& D, cudaStream_t st,
+                                   bool chained = false);
 cudaError_t launch_mocca_bp(const GeomC& C, const ExcTable& E, const RayRec* rec, const ViewF* views,
-                            const StepParams& P, const SolveD& D, cudaStream_t st, const FpTables* T = nullptr);
+                            const StepParams& P, const SolveD& D, cudaStream_t st, const FpTables* T = nullptr,
+                            bool chained = false);
 cudaError_t launch_dtpl_reduce(const double* part, int n, double* out, cudaStream_t st);
 // View split of one iteration: the back-projection of the views [v0, v1) into
 // the nine per-pixel channels chan [9][P] (no primal step), and the primal step
