@@ -53,11 +53,12 @@ void free_ctx(osscir_ctx* h) {
     if (h->join) cudaEventDestroy(h->join);
     void* ptrs[] = {h->scratch, h->rec,     h->r64,    h->views,     h->chord,    h->exc_off,    h->exc_ent,  h->s4,
                     h->N4,      h->mu,     h->mu_in,     h->g,        h->c,          h->y,        h->x,
-                    h->xbar,    h->xo,     h->dtpl_part, h->dtpl_out, h->bad_counts, h->model,    h->fwd_unit,
+                    h->xbar,    h->xo,     h->dtpl_part, h->dtpl_out, h->model,    h->fwd_unit,
                     h->fwd_cnt, h->fwd_k0, h->fwd_w, h->fwd_d, h->bp_span, h->bp_unit, h->bp_w,
                     h->bp_slot, h->bp_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    if (h->report) cudaFreeHost(h->report);
     delete h;
 }
 
@@ -282,8 +283,9 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     CK(dalloc(&h->x, P));
     CK(dalloc(&h->xbar, 2 * (size_t)P));   // row-major, then the column-major copy
     CK(dalloc(&h->dtpl_part, h->n_part));
-    CK(dalloc(&h->dtpl_out, 2));
-    CK(dalloc(&h->bad_counts, 2));
+    CK(dalloc(&h->dtpl_out, 3));
+    h->bad_counts = reinterpret_cast<int*>(h->dtpl_out + 2);
+    CK(cudaMallocHost(reinterpret_cast<void**>(&h->report), sizeof *h->report));
     if (h->inner > 1) CK(dalloc(&h->model, (size_t)kModelStride * L));
     CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&h->side_stream, cudaStreamNonBlocking));
@@ -747,13 +749,11 @@ osscir_status osscir_reconstruct(osscir_t h, const float* c_host, int n_iters, f
         xs = h->xo;
     }
     CK(cudaMemcpyAsync(maps_out_host, xs, sizeof(float4) * h->P, cudaMemcpyDeviceToHost, st));
-    double d = 0.0;   // D_TPL at the last expansion point (the value the iterations computed)
-    int kerr = 0;
-    if (n_iters > 0) CK(cudaMemcpyAsync(&d, h->dtpl_out + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&kerr, h->bad_counts + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->report, h->dtpl_out, sizeof *h->report, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (kerr) return OSSCIR_E_CUDA;
-    if (!std::isfinite(d)) return OSSCIR_E_DIVERGED;
+    if (h->report->bad[1]) return OSSCIR_E_CUDA;
+    // D_TPL at the last expansion point (the value the iterations computed)
+    if (n_iters > 0 && !std::isfinite(h->report->dtpl[1])) return OSSCIR_E_DIVERGED;
     return OSSCIR_OK;
 }
 
@@ -801,12 +801,11 @@ osscir_status osscir_dtpl(osscir_t h, int which, double* out, void* stream) {
         CK(launch_counts(h->gc, h->exc(), h->rec, h->spec(), h->x, nullptr, h->c, h->dtpl_part, st));
         CK(launch_dtpl_reduce(h->dtpl_part, h->n_part, h->dtpl_out, st));
     }
-    int bad[2] = {0, 0};
-    CK(cudaMemcpyAsync(out, h->dtpl_out + which, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(bad, h->bad_counts, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->report, h->dtpl_out, sizeof *h->report, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (bad[1]) return OSSCIR_E_CUDA;
-    if (bad[0]) return OSSCIR_E_INVALID;
+    *out = h->report->dtpl[which];
+    if (h->report->bad[1]) return OSSCIR_E_CUDA;
+    if (h->report->bad[0]) return OSSCIR_E_INVALID;
     if (!std::isfinite(*out)) return OSSCIR_E_DIVERGED;
     return OSSCIR_OK;
 }

@@ -42,9 +42,16 @@ struct osscir_ctx {
     float4* x = nullptr;
     float4* xbar = nullptr;
     double* dtpl_part = nullptr;
-    double* dtpl_out = nullptr;   // [0]: at x (on request), [1]: at the last expansion point
-    int* bad_counts = nullptr;    // [0]: set by the check of the counts osscir_set_counts loads (0: valid);
+    double* dtpl_out = nullptr;   // [0]: at x (on request), [1]: at the last expansion point; bad_counts follows
+    int* bad_counts = nullptr;    // (in the same allocation) [0]: set by the check of the counts osscir_set_counts loads (0: valid);
                                   // [1]: set by a kernel whose bounded wait for its own copies ran out
+    // page-locked copy of dtpl_out and bad_counts: one asynchronous copy instead of two that
+    // each hold the host until the device is done
+    struct Report {
+        double dtpl[2];
+        int bad[2];
+    };
+    Report* report = nullptr;
     int n_part = 0;
     int exp_model = 0;   // counts model: 0 softexp (Eq. finalModel), 1 exp (Eq. fullModel)
     int iter = 0;
