@@ -73,15 +73,15 @@ FP32_LANES_PER_SM, SCHEDULERS_PER_SM, L1_BYTES_PER_CLK_PER_SM, L1_WAVEFRONTS_PER
 # elapsed SM cycles x the capturing GPU's SMs).  Valid only for that workload and for
 # the kernel sources they were taken on (source_sha, see _source_sha).
 NCU_WORKLOAD = "medium_256"
-_SHA = "b6ce277f6d9a2514"
+_SHA = "dea47b757b48fa99"
 NCU_COUNTS = {
-    "k_fp_proj": {"dram_bytes": 363276544 + 4203520, "warp_instructions": 41112016,
-                  "l1_wavefronts": 16519622, "source_sha": _SHA},
-    "k_mocca_ray": {"dram_bytes": 23119360 + 892672, "warp_instructions": 93367586,
-                    "l1_wavefronts": 8975038, "source_sha": _SHA},
+    "k_fp_proj": {"dram_bytes": 353642496 + 5072640, "warp_instructions": 15558048,
+                  "l1_wavefronts": 16744000, "source_sha": _SHA},
+    "k_mocca_ray": {"dram_bytes": 14810112 + 382208, "warp_instructions": 91877016,
+                    "l1_wavefronts": 8824000, "source_sha": _SHA},
     # the back-projection's two launches: k_fpb_bp and k_fpb_finish
-    "k_fpb_bp": {"dram_bytes": 436254720 + 4344320 + 19977984, "warp_instructions": 68896272 + 1998848,
-                 "l1_wavefronts": 26924140 + 264357, "source_sha": _SHA},
+    "k_fpb_bp": {"dram_bytes": 459161344 + 9107200 + 19988992, "warp_instructions": 72630248 + 2023424,
+                 "l1_wavefronts": 21878000 + 292000, "source_sha": _SHA},
 }
 
 
@@ -376,11 +376,12 @@ def run_gpu(args):
         # footprint tables: the projections stream them.  Algorithmic HBM bytes per
         # launch: forward 6 B per footprint pair (weight, 16-bit pixel step) + xbar read
         # (16 B per pixel) + g written and the pair count and first pixel read (24 B per
-        # ray); back-projection 6 B per pair (weight, stage slot) + the view groups'
-        # channel sums written and read (2 x 36 B per pixel and group) + x read and
-        # written, xbar and its column-major copy written (64 B per pixel)
+        # ray); back-projection 4 B per pair (its weight; the slot steps, a byte per ray and
+        # pair of pixels, are not counted) + the view groups' channel sums written and
+        # read (2 x 36 B per pixel and group) + x read and written, xbar and its
+        # column-major copy written (64 B per pixel)
         names = ("k_fp_proj", "k_mocca_ray", "k_fpb_bp")
-        alg = (6.0 * nnz + 16.0 * P + 24.0 * L, None, 6.0 * nnz + 72.0 * G * P + 64.0 * P)
+        alg = (6.0 * nnz + 16.0 * P + 24.0 * L, None, 4.0 * nnz + 72.0 * G * P + 64.0 * P)
     else:
         names = ("k_mocca_proj", "k_mocca_ray", "k_mocca_bp")
         alg = (None, None, None)
