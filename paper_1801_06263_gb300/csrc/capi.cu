@@ -249,7 +249,9 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     C.scale = (float)(g->sdd_mm / g->bin_mm);
     C.mid = (float)(0.5 * (g->n_bins - 1));
     C.margin_mm = (float)(1e-5 * r_img + 1e-3 * g->pixel_mm);
-    C.margin_bins = 0.01f;
+    C.margin_bins = (float)(0.01 + 0x1p-22 * g->n_bins);
+    C.slack_num = (float)(48 * 0x1p-24 * r_img);
+    C.slack_den = (float)(48 * 0x1p-24 * g->sid_mm);
     h->params.lambda = (float)pa->lambda;
     h->params.model = pa->model;
     h->params.spc = pa->spc == 2 ? 1 : pa->spc;   // mu-PC runs the diagonal SPC in its basis

@@ -310,25 +310,36 @@ struct GeomC {
     float sid, scale, mid;   // scale = sdd / bin_mm, mid = (n_bins - 1) / 2
     float margin_mm;         // candidate margin for the ray-driven enumeration
     float margin_bins;       // candidate margin for the pixel-driven enumeration
+    float slack_num, slack_den;   // FP32 error bounds of its lengths across and along the view (box_bin_range)
 };
 
 // Bins whose centre ray can cross the box of half extents (hx, hy) around (X, Y) in a
-// view (a superset of its shadow, in FP32 with a margin; x_weight decides).  With
-// num = q . e_u and den = sid - q . e at the centre, a corner at (+-hx, +-hy) from it
-// moves beta by scale (dx (c num - s den) + dy (c den + s num)) / (den den'), den' the
-// corner's own den, so half the shadow's width is at most
-// scale (hx |c num - s den| + hy |c den + s num|) / (den min den').  One point and two
-// divisions instead of the four corners': about 25 instructions instead of 55 for
-// each of the pixel-views that the pixel-driven kernels visit; the bound is wider
+// view: a superset of its shadow (x_weight decides), so that a box that holds another's
+// has a range that holds every bin the other meets.  With r = (q . e_u) / den and
+// den = sid - q . e at the centre, a corner at (+-hx, +-hy) from it moves beta by
+// scale (dx (c r - s) + dy (c + s r)) / den', den' the corner's own den, so half the
+// shadow's width is at most scale (hx |c r - s| + hy |c + s r|) / min den'.  One point
+// and two divisions instead of the four corners': about 25 instructions instead of 55
+// for each of the pixel-views that the pixel-driven kernels visit; the bound is wider
 // than the shadow by a factor h / den at most (0.1 % for a pixel at 256 x 256).
+// FP32 error, in rounding units u = 2^-24, with R the image's half diagonal (|q| <= R <
+// sid): q . e_u is within 8 R u, den within 11 sid u, so r with its division's 2 ulp
+// within (8 R + 22 sid |r|) u / den; carried through reach as well (its slope in r is
+// den - den_min) and with reach's own roundings, beta +- half is within
+// 34 scale (R + sid |r|) u / den_min.  slack_num + slack_den |r| = 48 (R + sid |r|) u in
+// reach covers this, slack_den den_min's own error and margin_bins the sums with mid.
+// A fixed margin of 0.01 bins alone does not: 65535 bins around 4096 x 4096 pixels, or
+// 8192 bins and a source just outside a 512 x 512 image, lost bins of the exact shadow.
+// Only ratios of lengths are formed, so any unit of length will do.
 __device__ __forceinline__ void box_bin_range(const GeomC& C, const ViewF& V, float X, float Y, float hx, float hy,
                                               int& blo, int& bhi) {
     const float num = fmaf(V.c, Y, -V.s * X), den = C.sid - fmaf(V.c, X, V.s * Y);
-    const float den_min = fmaxf(den - fmaf(hx, fabsf(V.c), hy * fabsf(V.s)), 1e-6f * den);
-    const float reach = fmaf(hx, fabsf(fmaf(V.c, num, -V.s * den)), hy * fabsf(fmaf(V.c, den, V.s * num)));
-    // __fdividef is within 2 ulp; the margin covers it
-    const float beta = fmaf(C.scale, __fdividef(num, den), C.mid);
-    const float half = fmaf(C.scale, __fdividef(reach, den * den_min), C.margin_bins);
+    const float den_min = fmaxf(den - fmaf(hx, fabsf(V.c), fmaf(hy, fabsf(V.s), C.slack_den)), 1e-6f * den);
+    const float r = __fdividef(num, den);
+    const float reach = fmaf(hx, fabsf(fmaf(V.c, r, -V.s)),
+                             fmaf(hy, fabsf(fmaf(V.s, r, V.c)), fmaf(C.slack_den, fabsf(r), C.slack_num)));
+    const float beta = fmaf(C.scale, r, C.mid);
+    const float half = fmaf(C.scale, __fdividef(reach, den_min), C.margin_bins);
     blo = max(0, -sat_floor(half - beta));
     bhi = min(C.n_bins - 1, sat_floor(beta + half));
 }
