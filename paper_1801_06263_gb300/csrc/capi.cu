@@ -417,7 +417,7 @@ osscir_status build_tables(osscir_ctx* h) {
     // back-projection (blocked): per tile and view the bins that can meet it; the chunk
     // size (views per staged chunk) whose two stage buffers fit; the units of each
     // (block, warp, chunk) and their prefix sum; then the entries
-    if (e == cudaSuccess) e = dalloc(&h->bp_span, (size_t)n_t * C.n_views);
+    if (e == cudaSuccess) e = dalloc(&h->bp_span, bt_spans(C.grid.n, C.n_views));
     if (e == cudaSuccess) e = launch_fpb_span(C, h->views, G, h->bp_span, dev(&stat.most[0]), st);
     if (e == cudaSuccess) e = read_stat();
     // forward: the pairs; one more unit than the table has (it is loaded ahead)

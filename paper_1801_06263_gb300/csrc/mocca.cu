@@ -1625,10 +1625,10 @@ __device__ __forceinline__ void chunk_views(int n_views, int g, int G, int chunk
 
 // Table pass 0: per tile and view the bins that can meet the tile, tlo | span << 16.
 __global__ void __launch_bounds__(256) k_fpb_span(GeomC C, const ViewF* views, uint32_t* span) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, n = C.grid.n;
-    const int ntx = (n + kBTX - 1) / kBTX, n_t = ntx * ((n + kBTY - 1) / kBTY);
-    if (i >= n_t * C.n_views) return;
-    const int t = i / C.n_views, v = i % C.n_views;
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = C.grid.n, ntx = (n + kBTX - 1) / kBTX, n_t = ntx * ((n + kBTY - 1) / kBTY);
+    if (i >= (size_t)n_t * C.n_views) return;
+    const int t = (int)(i / C.n_views), v = (int)(i % C.n_views);
     const int ix = (t % ntx) * kBTX, iy = (t / ntx) * kBTY;
     const float X0 = grid_plane(C.grid, ix), X1 = grid_plane(C.grid, min(n, ix + kBTX));
     const float Y0 = grid_plane(C.grid, iy), Y1 = grid_plane(C.grid, min(n, iy + kBTY));
@@ -2403,7 +2403,7 @@ cudaError_t launch_fp_fwd_fill(const GeomC& C, const ExcTable& E, const RayRec* 
     return cudaGetLastError();
 }
 cudaError_t launch_fpb_span(const GeomC& C, const ViewF* views, int G, uint32_t* span, int* most, cudaStream_t st) {
-    k_fpb_span<<<blocks(bt_tiles(C.grid.n) * C.n_views, 256), 256, 0, st>>>(C, views, span);
+    k_fpb_span<<<thread_blocks(bt_spans(C.grid.n, C.n_views), 256), 256, 0, st>>>(C, views, span);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_fpb_most<<<blocks(bt_tiles(C.grid.n) * G, 128), 128, 0, st>>>(C, span, G, most);

@@ -68,6 +68,10 @@ constexpr int kBpMaxThreads = 512;                    // kBpPix x up to 8 view g
 constexpr int kBTX = 16, kBTY = 16, kBTThreads = kBTX * kBTY / 2, kBTWarps = kBTThreads / 32, kBTMaxChunk = 16;
 constexpr int kBTSlots = 396;   // slots of a stage buffer (two of 36 bytes a slot: 28 KB, seven blocks per SM)
 inline int bt_tiles(int n) { return ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / kBTY); }
+// Entries of bp_span: one per tile and view (2^31 for 8192 x 8192 pixels and 8192 views).
+inline size_t bt_spans(int n, int n_views) { return (size_t)bt_tiles(n) * n_views; }
+// Blocks of t threads for n of them, one each.
+inline unsigned thread_blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 // Footprint tables of one geometry: the pairs (l, k) of X with their weights,
 // in the order each projector visits them.

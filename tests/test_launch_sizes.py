@@ -1,0 +1,37 @@
+"""Launch sizes of the footprint tables' passes (csrc/osscir_launch.h) at the largest
+accepted geometries, from the host helpers that the launchers use (a small program
+compiled here; no GPU): the tile-view pairs of 8192 x 8192 pixels pass 2^31 at 8192 views
+and 2^32 above 16384."""
+import subprocess
+
+import pytest
+
+from paper_1801_06263_gb300 import build
+
+SOURCE = """
+#include <cstdio>
+#include <cstdlib>
+#include "osscir_launch.h"
+int main(int, char** a) {
+    const size_t s = osscir::bt_spans(atoi(a[1]), atoi(a[2]));
+    printf("%zu %u", s, osscir::thread_blocks(s, 256));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    d = tmp_path_factory.mktemp("launch_sizes")
+    (d / "p.cu").write_text(SOURCE)
+    out = str(d / "p")
+    subprocess.run([build._nvcc(), "-std=c++17", "--expt-relaxed-constexpr", "-I", build.CSRC, "-o", out, str(d / "p.cu")],
+                   check=True, capture_output=True)
+    return out
+
+
+@pytest.mark.parametrize("n,views", [(1, 1), (256, 512), (8191, 8192), (8192, 8192), (8192, 16385), (8192, 100000)])
+def test_span_pass_covers_every_tile_and_view(program, n, views):
+    spans, blocks = map(int, subprocess.run([program, str(n), str(views)], check=True, capture_output=True,
+                                            text=True).stdout.split())
+    want = ((n + 15) // 16) ** 2 * views
+    assert spans == want and blocks == (want + 255) // 256 < 2 ** 31
