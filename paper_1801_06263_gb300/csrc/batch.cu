@@ -140,6 +140,7 @@ void build_items(const std::vector<osscir_ctx*>& ctx, int first, int n, int k, c
 struct Plan {
     int branches = 1;
     bool tables = false;              // the back-projection streams every solve's tables
+    int slots = 0;                    // their largest bp_slots
     std::vector<osscir_ctx*> order;   // descriptor order
     int first[kMaxBranches] = {0, 0, 0, 0}, count[kMaxBranches] = {0, 0, 0, 0};
     size_t off[kMaxBranches][4] = {};
@@ -169,6 +170,8 @@ void make_plan(const std::vector<osscir_ctx*>& ctx, const osscir_batch_config& c
         p.count[b] = (int)p.order.size() - p.first[b];
     }
     p.tables = all_tables(ctx);
+    p.slots = 0;
+    for (const osscir_ctx* h : ctx) p.slots = std::max(p.slots, h->bp_slots);
     size_t bytes = sizeof(SolveDesc) * n;
     std::vector<int2> lists[kMaxBranches][4];
     for (int b = 0; b < p.branches; ++b)
@@ -203,7 +206,7 @@ cudaError_t launch_branch_kernel(const Plan& p, const char* dev, int b, int k, c
     if (k == 0) return launch_batch_proj(d, it, n, c.proj_views, c.proj_grid, st);
     if (k == 1) return launch_batch_ray(d, it, n, c.ray_grid, st);
     if (p.tables)
-        return launch_batch_fpb(d, it, n, plan_items(p, dev, b, 3), p.n_items[b][3], c.bp_grid, st);
+        return launch_batch_fpb(d, it, n, plan_items(p, dev, b, 3), p.n_items[b][3], c.bp_grid, p.slots, st);
     return launch_batch_bp(d, it, n, c.bp_tile_x, c.bp_grid, st);
 }
 
@@ -467,7 +470,7 @@ osscir_status autotune(osscir_batch* b) {
     const int threads[3] = {32 * kDefault.proj_views, kFwdThreads, tables ? kBTThreads : kBpMaxThreads};
     for (int k = 0; k < 3 && s == OSSCIR_OK; ++k) {
         int per_sm = 0;
-        e = (k == 2 && tables) ? batch_resident_ctas(3, threads[k], &per_sm)
+        e = (k == 2 && tables) ? batch_resident_ctas(b->plan.slots > kBTSlots ? 4 : 3, threads[k], &per_sm)
                                : batch_resident_ctas(k, threads[k], &per_sm);
         if (e != cudaSuccess) {
             s = from_cuda(e);

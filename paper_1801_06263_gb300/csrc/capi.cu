@@ -428,8 +428,9 @@ osscir_status build_tables(osscir_ctx* h) {
     if (e == cudaSuccess)
         e = launch_fp_fwd_fill(C, h->exc(), h->rec, h->fwd_unit, h->fwd_w, h->fwd_d, h->fwd_k0, dev(&stat.bad), st);
     int chunk = 0;
+    h->bp_slots = stat.most[0] <= kBTSlots ? kBTSlots : kBTSlotsFine;
     for (int i = kBTSizes - 1; i >= 0 && !chunk && C.n_bins <= 65535; --i)   // bp_span holds a bin in 16 bits
-        if (stat.most[i] <= kBTSlots) chunk = bt_size(i);
+        if (stat.most[i] <= h->bp_slots) chunk = bt_size(i);
     if (e == cudaSuccess && chunk > 0) {
         h->bp_groups = G;
         h->bp_chunk = chunk;

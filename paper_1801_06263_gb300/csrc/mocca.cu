@@ -1782,10 +1782,13 @@ __global__ void __launch_bounds__(kBTThreads) k_fpb_fill(GeomC C, ExcTable E, co
     }
 }
 
-// A stage buffer of kBTSlots slots: s0 (b, S00) at its start, s1 (S01, S02, S11, S12) at
-// kBTStageS1 and s22 at kBTStageS22, addressed with 32-bit shared addresses (through
-// generic pointers the reads of a row cost twice the instructions).
-constexpr uint32_t kBTStageS1 = 16 * kBTSlots, kBTStageS22 = 32 * kBTSlots, kBTStage = 36 * kBTSlots;
+// A stage buffer of SLOTS slots: s0 (b, S00) at its start, s1 (S01, S02, S11, S12) at
+// kS1 and s22 at kS22, addressed with 32-bit shared addresses (through generic pointers
+// the reads of a row cost twice the instructions).
+template <int SLOTS>
+struct Stage {
+    static constexpr uint32_t kS1 = 16 * SLOTS, kS22 = 32 * SLOTS, kBytes = 36 * SLOTS;
+};
 __device__ __forceinline__ float4 lds4(uint32_t a) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
@@ -1802,7 +1805,7 @@ __device__ __forceinline__ void sts1(uint32_t a, float v) { asm volatile("st.sha
 // asynchronously: warp w copies views u0 + w, u0 + w + kBTWarps, ..., lane i bin i of
 // the view's run.  sp: lane i's bp_span of view u0 + i (0 beyond u1).  PARTIAL: the rays
 // of views outside [V0, V1) are staged as zeros, so they add nothing.
-template <bool PARTIAL>
+template <bool PARTIAL, int SLOTS>
 __device__ __forceinline__ void stage_views(const GeomC& C, const RaySteps& steps, uint32_t sp, int u0, int u1, int V0,
                                             int V1, uint32_t buf) {
     const int lane = threadIdx.x & 31;
@@ -1819,17 +1822,17 @@ __device__ __forceinline__ void stage_views(const GeomC& C, const RaySteps& step
         const size_t l0 = (size_t)(u0 + i) * C.n_bins + (si & 0xffffu);
         const bool out = PARTIAL && (u0 + i < V0 || u0 + i >= V1);
         for (int p = lane; p < n; p += 32) {
-            const uint32_t a = buf + 16u * (oi + p), z = buf + kBTStageS22 + 4u * (oi + p);
+            const uint32_t a = buf + 16u * (oi + p), z = buf + Stage<SLOTS>::kS22 + 4u * (oi + p);
             const size_t l = l0 + p;
             if (out) {
                 for (int j = 0; j < 4; ++j) {
                     sts1(a + 4 * j, 0.f);
-                    sts1(a + kBTStageS1 + 4 * j, 0.f);
+                    sts1(a + Stage<SLOTS>::kS1 + 4 * j, 0.f);
                 }
                 sts1(z, 0.f);
             } else {
                 cp_async16(a, steps.s0 + l);
-                cp_async16(a + kBTStageS1, steps.s1 + l);
+                cp_async16(a + Stage<SLOTS>::kS1, steps.s1 + l);
                 cp_async4(z, steps.s22 + l);
             }
         }
@@ -1867,7 +1870,7 @@ __device__ __forceinline__ Unit<WIDE> ld_unit(const float4* w, const uint32_t* s
 // ascending, bins ascending, nonzero weights only).  PARTIAL: only the rays of the
 // views [V0, V1) (one GPU's share of a split solve).  Every thread of the block must
 // call this (it contains block barriers).
-template <bool PARTIAL, bool WIDE>
+template <bool PARTIAL, bool WIDE, int SLOTS>
 __device__ __forceinline__ void fpb_sum_block(const GeomC& C, const FpTables& T, const RayRec* rec, int V0, int V1,
                                               float* part, int b, uint32_t smem) {
     const int G = T.bp_groups, t = b / G, g = b % G, tid = threadIdx.x, lane = tid & 31;
@@ -1900,7 +1903,7 @@ __device__ __forceinline__ void fpb_sum_block(const GeomC& C, const FpTables& T,
     auto stage = [&](int c, uint32_t sp) {
         int u0, u1;
         chunk_views(C.n_views, g, G, T.bp_chunk, c, u0, u1);
-        stage_views<PARTIAL>(C, steps, sp, u0, u1, V0, V1, smem + (c & 1) * kBTStage);
+        stage_views<PARTIAL, SLOTS>(C, steps, sp, u0, u1, V0, V1, smem + (c & 1) * Stage<SLOTS>::kBytes);
     };
     if (c_lo < c_hi) {
         const uint32_t* up = T.bp_unit + ((size_t)b * kBTWarps + (tid >> 5)) * nch;
@@ -1928,10 +1931,10 @@ __device__ __forceinline__ void fpb_sum_block(const GeomC& C, const FpTables& T,
                 l2_prefetch(T.bp_slot + (size_t)(WIDE ? 64 : 32) * q1, (WIDE ? 256u : 128u) * (q2 - q1));
             }
             // the addresses of the row's slot: its s0 (s1 at a constant distance) and its s22
-            uint32_t at = smem + (c & 1) * kBTStage, az = at + kBTStageS22;
+            uint32_t at = smem + (c & 1) * Stage<SLOTS>::kBytes, az = at + Stage<SLOTS>::kS22;
             const uint32_t at0 = at, az0 = az;
             auto row = [&](float w0, float w1) {
-                const float4 s0 = lds4(at), s1 = lds4(at + kBTStageS1);
+                const float4 s0 = lds4(at), s1 = lds4(at + Stage<SLOTS>::kS1);
                 const float z = lds1(az);
                 bp_accumulate_if(acc, w0, s0, s1, z);
                 bp_accumulate_if(acc + 9, w1, s0, s1, z);
@@ -1994,23 +1997,26 @@ __device__ __forceinline__ void fpb_sum_block(const GeomC& C, const FpTables& T,
     }
 }
 
-template <bool PARTIAL>
+template <bool PARTIAL, int SLOTS>
 __device__ __forceinline__ void fpb_block(const GeomC& C, const FpTables& T, const RayRec* rec, int V0, int V1,
                                           float* part, int b) {
-    __shared__ float4 stage[2 * kBTStage / 16];
+    __shared__ float4 stage[2 * Stage<SLOTS>::kBytes / 16];
     const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(stage));
-    if (T.bp_wide) fpb_sum_block<PARTIAL, true>(C, T, rec, V0, V1, part, b, sa);
-    else fpb_sum_block<PARTIAL, false>(C, T, rec, V0, V1, part, b, sa);
+    if (T.bp_wide) fpb_sum_block<PARTIAL, true, SLOTS>(C, T, rec, V0, V1, part, b, sa);
+    else fpb_sum_block<PARTIAL, false, SLOTS>(C, T, rec, V0, V1, part, b, sa);
 }
 
 // Seven resident blocks (72 registers, a handful of spilled words): 109 us at 256 x 256
 // with the step and 683 us at 512 x 512, against 115 and 707 with six; eight (64
 // registers) were slower.
-constexpr int kBTResident = 7;
-template <bool PARTIAL>
-__global__ void __launch_bounds__(kBTThreads, kBTResident) k_fpb_bp(GeomC C, FpTables T, const RayRec* rec, int V0, int V1,
-                                                       float* part) {
-    fpb_block<PARTIAL>(C, T, rec, V0, V1, part, blockIdx.x);
+// Fine detectors' larger stages leave five: 64 x 64 pixels seen by 2048 bins (100 views)
+// take 65 us, 186 without a table; 32 x 32 seen by 896 bins 59 and 160.
+template <int SLOTS>
+constexpr int kBTResident = SLOTS == kBTSlots ? 7 : 5;
+template <bool PARTIAL, int SLOTS>
+__global__ void __launch_bounds__(kBTThreads, kBTResident<SLOTS>)
+    k_fpb_bp(GeomC C, FpTables T, const RayRec* rec, int V0, int V1, float* part) {
+    fpb_block<PARTIAL, SLOTS>(C, T, rec, V0, V1, part, blockIdx.x);
 }
 
 // The view groups of pixel k added in group order (as bp_finish does), three groups'
@@ -2173,12 +2179,13 @@ __global__ void __launch_bounds__(kBatchProjMaxThreads) k_batch_proj(const Solve
 
 // Batched back-projection from the solves' blocked tables: item (solve, block b)
 // runs fpb_block.
-__global__ void __launch_bounds__(kBTThreads, kBTResident) k_batch_fpb_bp(const SolveDesc* __restrict__ sd,
-                                                             const int2* __restrict__ items, int n_items) {
+template <int SLOTS>
+__global__ void __launch_bounds__(kBTThreads, kBTResident<SLOTS>)
+    k_batch_fpb_bp(const SolveDesc* __restrict__ sd, const int2* __restrict__ items, int n_items) {
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
         const int2 w = __ldg(items + it);
         const SolveDesc& d = sd[w.x];
-        fpb_block<false>(d.C, d.T, d.rec, 0, d.C.n_views, d.T.bp_part, w.y);
+        fpb_block<false, SLOTS>(d.C, d.T, d.rec, 0, d.C.n_views, d.T.bp_part, w.y);
     }
 }
 
@@ -2355,7 +2362,8 @@ cudaError_t launch_mocca_ray_inner(const GeomC& C, RayRec* rec, const SolveD& D,
 template <bool PARTIAL>
 cudaError_t launch_fpb(const GeomC& C, const FpTables& T, const RayRec* rec, const StepParams& P, const SolveD& D,
                        int v0, int v1, float* chan, cudaStream_t st, bool chained = false) {
-    launch_iter(k_fpb_bp<PARTIAL>, bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, st, chained, C, T, rec, v0, v1, T.bp_part);
+    launch_iter(T.bp_slots == kBTSlots ? k_fpb_bp<PARTIAL, kBTSlots> : k_fpb_bp<PARTIAL, kBTSlotsFine>,
+                bt_tiles(C.grid.n) * T.bp_groups, kBTThreads, st, chained, C, T, rec, v0, v1, T.bp_part);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     launch_iter(k_fpb_finish<PARTIAL>, blocks(C.grid.n * C.grid.n, kFinishThreads), kFinishThreads, st, chained, C, P, D,
@@ -2470,9 +2478,10 @@ cudaError_t launch_batch_dtpl(const SolveDesc* sd, int n_solves, cudaStream_t st
 }
 
 cudaError_t launch_batch_fpb(const SolveDesc* sd, const int2* items, int n_items, const int2* fin_items,
-                             int n_fin, int grid, cudaStream_t st) {
+                             int n_fin, int grid, int slots, cudaStream_t st) {
     if (n_items > 0) {
-        k_batch_fpb_bp<<<grid > 0 ? grid : n_items, kBTThreads, 0, st>>>(sd, items, n_items);
+        (slots <= kBTSlots ? k_batch_fpb_bp<kBTSlots> : k_batch_fpb_bp<kBTSlotsFine>)
+            <<<grid > 0 ? grid : n_items, kBTThreads, 0, st>>>(sd, items, n_items);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -2485,7 +2494,8 @@ cudaError_t batch_resident_ctas(int kernel, int threads, int* per_sm) {
     switch (kernel) {
         case 0: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_proj, threads, 0);
         case 1: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_ray, threads, 0);
-        case 3: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_fpb_bp, threads, 0);
+        case 3: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_fpb_bp<kBTSlots>, threads, 0);
+        case 4: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_fpb_bp<kBTSlotsFine>, threads, 0);
         default: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_bp, threads, 0);
     }
 }

@@ -71,11 +71,11 @@ struct osscir_ctx {
     float4* bp_w = nullptr;   // null: the back-projection stays on the fly
     uint32_t* bp_slot = nullptr;
     float* bp_part = nullptr;
-    int bp_groups = 1, bp_chunk = 0, bp_nch = 0, bp_wide = 0;
+    int bp_groups = 1, bp_chunk = 0, bp_nch = 0, bp_wide = 0, bp_slots = 0;
     size_t fp_bytes = 0;
     osscir::FpTables fp() const {
         return osscir::FpTables{fwd_unit, fwd_cnt, fwd_k0,    fwd_w,    fwd_d,  bp_span,  bp_unit, bp_w,
-                                bp_slot, bp_part, bp_groups, bp_chunk, bp_nch, bp_wide};
+                                bp_slot, bp_part, bp_groups, bp_chunk, bp_nch, bp_wide, bp_slots};
     }
     const osscir::FpTables* fp_or_null() const { return fp_state == 1 ? &fp_tab : nullptr; }
     osscir::FpTables fp_tab{};

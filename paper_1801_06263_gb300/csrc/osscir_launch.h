@@ -67,6 +67,9 @@ constexpr int kBpMaxThreads = 512;                    // kBpPix x up to 8 view g
 // most kBTMaxChunk.
 constexpr int kBTX = 16, kBTY = 16, kBTThreads = kBTX * kBTY / 2, kBTWarps = kBTThreads / 32, kBTMaxChunk = 16;
 constexpr int kBTSlots = 396;   // slots of a stage buffer (two of 36 bytes a slot: 28 KB, seven blocks per SM)
+// The same for detectors so fine (more than about 24 bins per pixel column) that a tile's
+// bins in one view exceed kBTSlots (40 KB, five blocks per SM).
+constexpr int kBTSlotsFine = 564;
 inline int bt_tiles(int n) { return ((n + kBTX - 1) / kBTX) * ((n + kBTY - 1) / kBTY); }
 // Entries of bp_span: one per tile and view (2^31 for 8192 x 8192 pixels and 8192 views).
 inline size_t bt_spans(int n, int n_views) { return (size_t)bt_tiles(n) * n_views; }
@@ -87,7 +90,7 @@ inline unsigned thread_blocks(size_t n, int t) { return (unsigned)((n + t - 1) /
 //   bp_groups); the group's views (the split of k_mocca_bp) in chunks of
 //   bp_chunk views, bp_nch chunks per group.  bp_span[t n_views + u] = tlo | span << 16:
 //   the bins that can meet the tile in view u.  A chunk's rays, view after view (ray
-//   (u, tlo + i)), are its stage slots, at most kBTSlots of them.  A thread has two
+//   (u, tlo + i)), are its stage slots, at most bp_slots of them.  A thread has two
 //   pixels, (ix, iy) and (ix, iy + 1); in a view it has one entry per bin from the
 //   first to the last that meets either, with the weights of both (0 where the ray
 //   misses one).  The rows of a warp are aligned per view (view u takes as many rows
@@ -112,6 +115,7 @@ struct FpTables {
     const uint32_t* bp_slot;
     float* bp_part;            // [bp_groups][9][P]
     int bp_groups, bp_chunk, bp_nch, bp_wide;
+    int bp_slots;              // kBTSlots or kBTSlotsFine
 };
 // View groups per pixel for the MOCCA back-projection: enough threads to fill
 // the GPU several times over, at most 8, and at least one view per group.
@@ -237,11 +241,12 @@ cudaError_t launch_batch_bp(const SolveDesc* sd, const int2* items, int n_items,
                             cudaStream_t st);
 cudaError_t launch_batch_dtpl(const SolveDesc* sd, int n_solves, cudaStream_t st);
 // Back-projection of solves with footprint tables: items (solve, table block),
-// then fin_items (solve, block of 256 pixels) for the group sums and a7.
+// then fin_items (solve, block of 256 pixels) for the group sums and a7; slots: the
+// largest bp_slots of the solves.
 cudaError_t launch_batch_fpb(const SolveDesc* sd, const int2* items, int n_items, const int2* fin_items,
-                             int n_fin, int grid, cudaStream_t st);
+                             int n_fin, int grid, int slots, cudaStream_t st);
 // Resident CTAs per SM of a batched kernel (0 projection, 1 ray, 2 back-projection
-// on the fly, 3 back-projection from tables).
+// on the fly, 3 back-projection from tables of at most kBTSlots, 4 of kBTSlotsFine slots).
 cudaError_t batch_resident_ctas(int kernel, int threads, int* per_sm);
 
 }  // namespace osscir
