@@ -248,6 +248,7 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     C.sid = (float)g->sid_mm;
     C.scale = (float)(g->sdd_mm / g->bin_mm);
     C.mid = (float)(0.5 * (g->n_bins - 1));
+    CK(cudaDeviceGetAttribute(&C.sms, cudaDevAttrMultiProcessorCount, h->device));
     C.margin_mm = (float)(1e-5 * r_img + 1e-3 * g->pixel_mm);
     C.margin_bins = (float)(0.01 + 0x1p-22 * g->n_bins);
     C.slack_num = (float)(48 * 0x1p-24 * r_img);

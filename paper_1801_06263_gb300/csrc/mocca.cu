@@ -932,10 +932,10 @@ __device__ __forceinline__ double ray_step(const GeomC& C, RayRec* rec, const Sp
 // four for five windows (128 registers; 0.136 ms against 0.152 ms with three).
 // FEW: a grid of at most three blocks per SM has registers to spare and too few warps to
 // hide the spectral table's L2 latency, so eight energies' loads are in flight at once
-// (168 registers, no spills): 64 x 64 (128 blocks) 54 -> 42 us after an L2 flush, an
-// iteration 71 -> 66 us; 128 x 128 with 180 views (270 blocks) 62 -> 49 and 89 -> 84 us;
-// 630 blocks of 300 x 300 were 9 % slower with it.
-constexpr unsigned kRayFewBlocks = 3 * 152;
+// (168 registers, no spills, three resident blocks): 64 x 64 (128 blocks) 54 -> 42 us
+// after an L2 flush, an iteration 71 -> 66 us; 270 blocks 41 -> 29 us and 450, the last
+// of one wave, 41 -> 31, but 558 blocks, a second wave, 43 -> 54 and 630 45 -> 54.
+constexpr int kRayFewPerSm = 3;
 template <bool KEEP, int W, bool CURV, bool FEW>
 __global__ void __launch_bounds__(kFwdThreads, FEW ? 3 : (W == 4 ? 5 : 4)) k_mocca_ray(GeomC C, RayRec* rec, SpecD S,
                                                                          StepParams P, SolveD D, int v0, int v1) {
@@ -1566,9 +1566,10 @@ __device__ __forceinline__ void fp_proj_ray(const FpTables& T, const SolveD& D, 
 // Loads in flight count for more than resident warps: with four units per trip and the
 // registers for it 86 us at 256 x 256 (six resident blocks 93, eight 95, ten 99; 109
 // before).  Eight units per trip take a 64 x 64 image's 128 blocks 15 instead of
-// 18.5 us and 630 blocks of 300 x 300 56 instead of 63 us, but 256 x 256's 2048 blocks
-// 98 us: kFwdFewBlocks lies between.
-constexpr unsigned kFwdFewBlocks = 6 * 152;   // six blocks per SM
+// 18.5 us, 450 blocks 29 instead of 31, 630 33 instead of 37 and 750 the same 39, but
+// 900 blocks 43 instead of 41 and 256 x 256's 2048 100 instead of 84: the line is at
+// five blocks per SM.
+constexpr int kFwdFewPerSm = 5;
 template <int UN>
 __global__ void __launch_bounds__(kFwdThreads, UN > 4 ? 3 : 4) k_fp_proj(GeomC C, FpTables T, SolveD D, int v0, int v1) {
     const int bx = centre_out(blockIdx.y, gridDim.y);
@@ -2309,7 +2310,7 @@ cudaError_t launch_mocca_proj(const GeomC& C, const ExcTable& E, const RayRec* r
                               cudaStream_t st, int v0, int v1, const FpTables* T, bool chained) {
     if (v1 < 0) v1 = C.n_views;
     const dim3 fg = fwd_grid(C.n_bins, v1 - v0);
-    if (T && fg.x * fg.y <= kFwdFewBlocks) launch_iter(k_fp_proj<8>, dim3(fg.y, fg.x), kFwdThreads, st, chained, C, *T, D, v0, v1);
+    if (T && few_blocks(fg, kFwdFewPerSm, C.sms)) launch_iter(k_fp_proj<8>, dim3(fg.y, fg.x), kFwdThreads, st, chained, C, *T, D, v0, v1);
     else if (T) launch_iter(k_fp_proj<4>, dim3(fg.y, fg.x), kFwdThreads, st, chained, C, *T, D, v0, v1);
     else k_mocca_proj<<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, E, rec, D, v0, v1);
     return cudaGetLastError();
@@ -2319,7 +2320,7 @@ template <bool KEEP, int W, bool CURV>
 void launch_ray_grid(const GeomC& C, RayRec* rec, const SpecD& S, const StepParams& P, const SolveD& D, int v0, int v1,
                      cudaStream_t st, bool chained) {
     const dim3 grid = fwd_grid(C.n_bins, v1 - v0);
-    const auto kernel = grid.x * grid.y <= kRayFewBlocks ? k_mocca_ray<KEEP, W, CURV, true> : k_mocca_ray<KEEP, W, CURV, false>;
+    const auto kernel = few_blocks(grid, kRayFewPerSm, C.sms) ? k_mocca_ray<KEEP, W, CURV, true> : k_mocca_ray<KEEP, W, CURV, false>;
     launch_iter(kernel, grid, kFwdThreads, st, chained, C, rec, S, P, D, v0, v1);
 }
 

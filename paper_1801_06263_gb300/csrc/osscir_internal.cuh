@@ -310,6 +310,7 @@ struct GeomC {
     float sid, scale, mid;   // scale = sdd / bin_mm, mid = (n_bins - 1) / 2
     float margin_mm;         // candidate margin for the ray-driven enumeration
     float margin_bins;       // candidate margin for the pixel-driven enumeration
+    int sms;                 // the device's SMs, for the launch rules that compare a grid with them
     float slack_num, slack_den;   // FP32 error bounds of its lengths across and along the view (box_bin_range)
 };
 

@@ -200,6 +200,8 @@ cudaError_t launch_mocca_apply(const GeomC& C, const StepParams& P, const SolveD
 inline dim3 fwd_grid(int n_bins, int n_views) {
     return dim3((n_bins + 31) / 32, (n_views + kFwdThreads / 32 - 1) / (kFwdThreads / 32));
 }
+// Whether a grid has at most `per_sm` blocks for each of the device's SMs.
+inline bool few_blocks(dim3 grid, int per_sm, int sms) { return (size_t)grid.x * grid.y <= (size_t)per_sm * sms; }
 // D_TPL partial sums: one per (view, group of 32 bins), i.e. per warp of the ray-driven kernels.
 inline int dtpl_partials(int n_bins, int n_views) { return n_views * ((n_bins + 31) / 32); }
 
