@@ -745,17 +745,33 @@ __device__ void ray_dual(const float (&al)[W][3], const float (&sinv)[W], const 
 
 // ------------------------------------------------------------------ fused MOCCA kernels
 
-// a1: line integrals of the three maps at the expansion point xbar.
+// a1: line integrals of the three maps at the expansion point xbar, computed on the fly.
+// FEW (at most kProjFewPerSm blocks per SM): two slabs a trip; larger grids hide the
+// gathers' latency with more warps, and one pair after the other (ray_weights), six
+// resident blocks per SM, takes fewer instructions.  270 blocks (128 x 128, 180
+// views) 58 us with FEW, 80 without; 1313 (389 x 389) 412 and 445; 1540 the same 137;
+// 2048 (256 x 256) 211 and 196; 8192 (512 x 512, 1024 views) 1276 and 1251.
+constexpr int kProjFewPerSm = 10;
+template <bool FEW>
 __device__ __forceinline__ void proj_ray(const GeomC& C, const ExcTable& E, const RayRec* rec, const SolveD& D,
                                          int l) {
-    const float4 gs = ray_line_sum(C, E, rec, D.xbar, l);
+    float4 gs;
+    if (FEW) {
+        gs = ray_line_sum(C, E, rec, D.xbar, l);
+    } else {
+        const float4 r0 = rec[l].r0, r1 = rec[l].r1;
+        LineSum acc;
+        ray_pixels(C, E, r0, r1.x, r1.y, l, [&](int k, float w) { acc.add(w, __ldg(D.xbar + k)); });
+        gs = acc.sum();
+    }
     D.g[l] = make_float4(gs.x, gs.y, gs.z, 0.f);
 }
 
-__global__ void __launch_bounds__(kFwdThreads, 8) k_mocca_proj(GeomC C, ExcTable E, const RayRec* rec, SolveD D,
-                                                                int v0, int v1) {
+template <bool FEW>
+__global__ void __launch_bounds__(kFwdThreads, FEW ? 5 : 6) k_mocca_proj(GeomC C, ExcTable E, const RayRec* rec,
+                                                                         SolveD D, int v0, int v1) {
     const int l = ray_in_views(C, centre_out(blockIdx.y, gridDim.y), blockIdx.x, kFwdThreads / 32, v0, v1);
-    if (l >= 0) proj_ray(C, E, rec, D, l);
+    if (l >= 0) proj_ray<FEW>(C, E, rec, D, l);
 }
 
 // a2-a5 and the per-ray half of a8: spectral model, curvature, dual step.
@@ -2173,7 +2189,7 @@ __global__ void __launch_bounds__(kBatchProjMaxThreads) k_batch_proj(const Solve
         const int l = ray_at(C, bx, w.y % nby, vb);
         if (l >= 0) {
             if (d.T.fwd_w) fp_proj_ray<4>(d.T, d.D, l, (l / C.n_bins) * nbx + bx);   // the solve's table
-            else proj_ray(C, d.E, d.rec, d.D, l);
+            else proj_ray<true>(C, d.E, d.rec, d.D, l);
         }
     }
 }
@@ -2312,7 +2328,9 @@ cudaError_t launch_mocca_proj(const GeomC& C, const ExcTable& E, const RayRec* r
     const dim3 fg = fwd_grid(C.n_bins, v1 - v0);
     if (T && few_blocks(fg, kFwdFewPerSm, C.sms)) launch_iter(k_fp_proj<8>, dim3(fg.y, fg.x), kFwdThreads, st, chained, C, *T, D, v0, v1);
     else if (T) launch_iter(k_fp_proj<4>, dim3(fg.y, fg.x), kFwdThreads, st, chained, C, *T, D, v0, v1);
-    else k_mocca_proj<<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, E, rec, D, v0, v1);
+    else if (few_blocks(fg, kProjFewPerSm, C.sms))
+        k_mocca_proj<true><<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, E, rec, D, v0, v1);
+    else k_mocca_proj<false><<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, E, rec, D, v0, v1);
     return cudaGetLastError();
 }
 
