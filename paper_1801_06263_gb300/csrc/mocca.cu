@@ -209,6 +209,14 @@ __device__ __forceinline__ int centre_out(int i, int n) {
     return (i & 1) ? c + (i + 1) / 2 : c - i / 2;
 }
 
+// The tile of block i of a one-dimensional grid in that order (a grid's second dimension
+// holds 65535 blocks: bin groups of at most 2 M bins, or views of at most 262140).
+__device__ __forceinline__ void tile_of_block(const GeomC& C, unsigned i, int& bx, int& by) {
+    const unsigned nby = (C.n_views + kFwdThreads / 32 - 1) / (kFwdThreads / 32);
+    bx = centre_out((int)(i / nby), (C.n_bins + 31) >> 5);
+    by = (int)(i % nby);
+}
+
 // x[k] where take is true, else unchanged.
 __device__ __forceinline__ void ldg_if(bool take, const float4* x, int k, float4& v) {
     asm("{\n\t.reg .pred p;\n\t"
@@ -295,8 +303,9 @@ __device__ __forceinline__ float4 ray_line_sum(const GeomC& C, const ExcTable& E
 
 __global__ void __launch_bounds__(kFwdThreads) k_forward4(GeomC C, ExcTable E, const RayRec* rec, const float4* x,
                                                           float4* g) {
-    const int bx = centre_out(blockIdx.y, gridDim.y);
-    const int l = ray_at(C, bx, blockIdx.x, kFwdThreads / 32);
+    int bx, by;
+    tile_of_block(C, blockIdx.x, bx, by);
+    const int l = ray_at(C, bx, by, kFwdThreads / 32);
     if (l >= 0) g[l] = ray_line_sum(C, E, rec, x, l);
 }
 
@@ -2301,7 +2310,7 @@ __global__ void k_xbar_columns(int n, float4* xbar) {
 cudaError_t launch_forward4(const GeomC& C, const ExcTable& E, const RayRec* rec, const float4* x, float4* g,
                             cudaStream_t st) {
     const dim3 fg = fwd_grid(C.n_bins, C.n_views);
-    k_forward4<<<dim3(fg.y, fg.x), kFwdThreads, 0, st>>>(C, E, rec, x, g);
+    k_forward4<<<fg.x * fg.y, kFwdThreads, 0, st>>>(C, E, rec, x, g);
     return cudaGetLastError();
 }
 
