@@ -334,7 +334,7 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     CK(cudaMemsetAsync(h->x, 0, sizeof(float4) * P, st));
     CK(cudaMemsetAsync(h->xbar, 0, sizeof(float4) * 2 * P, st));
     CK(cudaMemsetAsync(h->dtpl_out, 0, sizeof(double) * 2, st));
-    CK(cudaMemsetAsync(h->bad_counts, 0, 2 * sizeof(int), st));
+    CK(cudaMemsetAsync(h->bad_counts, 0, sizeof(int), st));
     CK(cudaStreamSynchronize(st));
     cudaFree(h->scratch);
     h->scratch = nullptr;
@@ -755,7 +755,6 @@ osscir_status osscir_reconstruct(osscir_t h, const float* c_host, int n_iters, f
     CK(cudaMemcpyAsync(maps_out_host, xs, sizeof(float4) * h->P, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(h->report, h->dtpl_out, sizeof *h->report, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (h->report->bad[1]) return OSSCIR_E_CUDA;
     // D_TPL at the last expansion point (the value the iterations computed)
     if (n_iters > 0 && !std::isfinite(h->report->dtpl[1])) return OSSCIR_E_DIVERGED;
     return OSSCIR_OK;
@@ -808,8 +807,7 @@ osscir_status osscir_dtpl(osscir_t h, int which, double* out, void* stream) {
     CK(cudaMemcpyAsync(h->report, h->dtpl_out, sizeof *h->report, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     *out = h->report->dtpl[which];
-    if (h->report->bad[1]) return OSSCIR_E_CUDA;
-    if (h->report->bad[0]) return OSSCIR_E_INVALID;
+    if (h->report->bad) return OSSCIR_E_INVALID;
     if (!std::isfinite(*out)) return OSSCIR_E_DIVERGED;
     return OSSCIR_OK;
 }

@@ -43,13 +43,12 @@ struct osscir_ctx {
     float4* xbar = nullptr;
     double* dtpl_part = nullptr;
     double* dtpl_out = nullptr;   // [0]: at x (on request), [1]: at the last expansion point; bad_counts follows
-    int* bad_counts = nullptr;    // (in the same allocation) [0]: set by the check of the counts osscir_set_counts loads (0: valid);
-                                  // [1]: set by a kernel whose bounded wait for its own copies ran out
+    int* bad_counts = nullptr;    // (in the same allocation) set by the check of the counts osscir_set_counts loads (0: valid)
     // page-locked copy of dtpl_out and bad_counts: one asynchronous copy instead of two that
     // each hold the host until the device is done
     struct Report {
         double dtpl[2];
-        int bad[2];
+        int bad;
     };
     Report* report = nullptr;
     int n_part = 0;
@@ -96,7 +95,7 @@ struct osscir_ctx {
     // float4 per ray of the window arrays c, y (and of the caller's counts): 1 for 4 windows, 2 for 5
     int wf4() const { return nw > 4 ? 2 : 1; }
     osscir::SolveD solve() const {
-        return osscir::SolveD{g, c, y, x, xbar, chord, dtpl_part, model, bad_counts ? bad_counts + 1 : nullptr};
+        return osscir::SolveD{g, c, y, x, xbar, chord, dtpl_part, model};
     }
 };
 

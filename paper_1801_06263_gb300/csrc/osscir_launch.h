@@ -49,7 +49,6 @@ struct SolveD {
     const float* chord; // [L] (X 1)_l
     double* dtpl_part;  // [fwd blocks]
     float4* model;      // [L][kModelStride] local models kept for nested MOCCA, or null
-    int* err;           // set to 1 by a kernel whose bounded wait for its own copies ran out (else untouched)
 };
 
 // Per-ray local model kept by an outer iteration of nested MOCCA (float4 slots):
