@@ -105,9 +105,10 @@ size_t estimate_bytes(const Config& c) {
     const size_t L = (size_t)c.geom.n_views * c.geom.n_bins, P = (size_t)c.geom.n * c.geom.n;
     const size_t per_ray = 64 + 32 + 4 + 4 + 16 + 16 + 8 * 4 / 128 + 2;   // records, FP64 rays, chord, offsets, c, y, partials
     const size_t mu_pc = c.params.spc == 2 ? P * 16 + 12 * c.nE : 0;   // the caller's curves and a maps buffer
-    // footprint tables: about 0.9 n footprint pairs per ray (0.82 n measured at 256 x 256), 6.9 bytes each
-    // in the forward table and 7.5 in the back-projection's (with the rows' padding), and the view
-    // groups' channel sums (at most 8 groups of 36 bytes per pixel)
+    // footprint tables: about 0.9 n footprint pairs per ray (0.82 to 0.85 n measured), 6.7 bytes each in
+    // the forward table and 8.0 in the back-projection's (256 x 256; 6.4 and 8.1 at 512 x 512), and the
+    // view groups' channel sums (at most 8 groups of 36 bytes per pixel).  Detectors of few bins or of
+    // odd groups of 32 take more (64 bins on 64 x 64 pixels 22 bytes in all): acquire sees to those
     const size_t tables = (size_t)(0.9 * c.geom.n * (double)L * 14.4) + P * 288 + L * 12;
     // x, and xbar with its column-major copy: 48 bytes per pixel
     return L * per_ray + P * 48 + (size_t)c.nE * c.geom.n_bins * 16 + c.geom.n_bins * 16 + 12 * c.nE +
@@ -177,16 +178,19 @@ struct osscir_server {
 Slot* osscir_server::acquire(Ticket* t) {
     for (Slot* s : slots)
         if (!s->running && s->key == t->key && s->cfg.same(t->cfg)) return s;
-    while (bytes_in_use + t->need > budget) {
+    auto release_idle = [&]() {
         Slot* victim = nullptr;
         for (Slot* s : slots)
             if (!s->running && (!victim || s->last_used < victim->last_used)) victim = s;
-        if (!victim) return nullptr;
+        if (!victim) return false;
         for (Group& g : groups) g.members.clear();   // a new context may reuse the address: re-form the batches
         slots.remove(victim);
         bytes_in_use -= victim->bytes;
         release_slot(victim);
-    }
+        return true;
+    };
+    while (bytes_in_use + t->need > budget)
+        if (!release_idle()) return nullptr;
     Slot* s = new (std::nothrow) Slot();
     if (!s) return nullptr;
     s->cfg = t->cfg;
@@ -206,6 +210,14 @@ Slot* osscir_server::acquire(Ticket* t) {
         return reinterpret_cast<Slot*>(-1);
     }
     s->bytes = s->ctx->bytes;
+    // where the estimate was low: room for the difference, or wait, now with the true
+    // size, until a running request ends (a request alone keeps what it was admitted with)
+    while (bytes_in_use + s->bytes > budget && release_idle()) {}
+    if (bytes_in_use > 0 && bytes_in_use + s->bytes > budget) {
+        t->need = std::min(s->bytes, budget);
+        release_slot(s);
+        return nullptr;
+    }
     bytes_in_use += s->bytes;
     slots.push_back(s);
     return s;
