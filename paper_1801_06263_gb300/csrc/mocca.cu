@@ -1,8 +1,9 @@
 // Per-iteration kernels of MOCCA with the m-block-diagonal SPC (Sec. 2) and the
 // plain projectors behind osscir_forward / osscir_backproject / osscir_simulate.
 //
-// One iteration is three launches (plus a tiny deterministic reduction):
-//   k_mocca_proj (ray-driven):  g = X xbar for the three maps;
+// One iteration is four launches from the footprint tables (three on the fly), and a
+// tiny deterministic reduction where D_TPL can be read:
+//   k_fp_proj, or on the fly k_mocca_proj (ray-driven):  g = X xbar for the three maps;
 //   k_mocca_ray (per ray):      the counts model
 //       of Eq. (finalModel) summed over energies (compensated), D_TPL of
 //       Eq. (DTPL), alpha_w = sum_i A_wi mu_i (K = alpha X, Eq. aeq), the per-ray
@@ -12,7 +13,8 @@
 //       y' = y - Sigma (W + Sigma)^-1 (y - r) (taken in an orthonormal basis of
 //       the range of alpha, see ray_dual), and the per-ray products b = alpha^T y'
 //       and S = sum_w alpha_w alpha_w^T / |alpha_w|.
-//   k_mocca_bp (pixel-driven):  v_k = sum_l X_lk b_l (= K^T y') and
+//   k_fpb_bp and k_fpb_finish, or on the fly k_mocca_bp (pixel-driven):
+//       v_k = sum_l X_lk b_l (= K^T y') and
 //       P_k = sum_l X_lk S_l (so T^-1_k = P_k / lambda, the m-block SPC), the
 //       3x3 solve (double-float), the primal step (optionally onto a box) and the
 //       extrapolation xbar' = 2 x' - x.
@@ -1305,7 +1307,7 @@ __device__ __forceinline__ void bp_partial_out(int P_, int k, bool valid, int pi
 
 // The end of a pixel's back-projection: group g of G stores its nine partial
 // sums in red ([G - 1][9][npix]); group 0 adds the others' in group order, then
-// solves T_k v = K^T y' in FP64 and takes the primal step.  Every thread of the
+// takes the primal step (pixel_step, in double-float).  Every thread of the
 // block must call this (it contains a block barrier).
 __device__ __forceinline__ void bp_finish(const GeomC& C, const StepParams& P, const SolveD& D, int ix, int iy,
                                           bool valid, int pix, int npix, int g, int G, float* red, float acc[9]) {
