@@ -94,6 +94,17 @@ def bp_view_groups(n_pixels, n_views):
     return G
 
 
+def projector_bytes(nnz, n_pixels, n_rays, groups):
+    """Algorithmic HBM bytes of the table projections of one iteration: forward 6 B per
+    footprint pair (weight, 16-bit pixel step) + xbar read (16 B per pixel) + g written and
+    the pair count and first pixel read (24 B per ray); back-projection 4 B per pair (its
+    weight; the slot steps, a byte per ray and pair of pixels, are not counted) + the view
+    groups' channel sums written and read (2 x 36 B per pixel and group) + x read and
+    written, xbar and its column-major copy written (64 B per pixel)."""
+    return (6.0 * nnz + 16.0 * n_pixels + 24.0 * n_rays,
+            4.0 * nnz + 72.0 * groups * n_pixels + 64.0 * n_pixels)
+
+
 def device_roofs(dev, sm_mhz):
     """Unit-count roofs of device `dev` at SM clock sm_mhz: FP32 TFLOP/s, warp
     instructions issued per second, L1-to-register TB/s; with how they were formed."""
@@ -373,15 +384,9 @@ def run_gpu(args):
     dev_bytes, table_bytes = _lib.osscir_memory(R.handle)
     G = bp_view_groups(P, w.geom.n_views)
     if table_bytes:
-        # footprint tables: the projections stream them.  Algorithmic HBM bytes per
-        # launch: forward 6 B per footprint pair (weight, 16-bit pixel step) + xbar read
-        # (16 B per pixel) + g written and the pair count and first pixel read (24 B per
-        # ray); back-projection 4 B per pair (its weight; the slot steps, a byte per ray and
-        # pair of pixels, are not counted) + the view groups' channel sums written and
-        # read (2 x 36 B per pixel and group) + x read and written, xbar and its
-        # column-major copy written (64 B per pixel)
         names = ("k_fp_proj", "k_mocca_ray", "k_fpb_bp")
-        alg = (6.0 * nnz + 16.0 * P + 24.0 * L, None, 4.0 * nnz + 72.0 * G * P + 64.0 * P)
+        fwd, bp = projector_bytes(nnz, P, L, G)
+        alg = (fwd, None, bp)
     else:
         names = ("k_mocca_proj", "k_mocca_ray", "k_mocca_bp")
         alg = (None, None, None)
@@ -683,8 +688,7 @@ def run_batched(args, rank):
     best_ms = min(default_ms, tuned_ms)
     # per kernel of the default configuration (one branch: one launch per kernel for all
     # solves), the algorithmic bytes of the plain path's table kernels summed over the
-    # solves: forward 6 B per footprint pair + 16 B per pixel + 24 B per ray; back-projection
-    # 6 B per pair + 72 B per pixel and view group + 64 B per pixel
+    # solves
     from paper_1801_06263_gb300 import osscir_footprint_rays
     fwd_bytes = bp_bytes = 0.0
     for R, w in zip(recs, ws):
@@ -692,8 +696,9 @@ def run_batched(args, rank):
         osscir_footprint_rays(R.handle, 0, w.geom.n_rays, 0, cnt, None, None)
         nnz = float(cnt.sum().item())
         Ps, Ls = w.geom.n_pixels, w.geom.n_rays
-        fwd_bytes += 6.0 * nnz + 16.0 * Ps + 24.0 * Ls
-        bp_bytes += 6.0 * nnz + 72.0 * bp_view_groups(Ps, w.geom.n_views) * Ps + 64.0 * Ps
+        fwd, bp = projector_bytes(nnz, Ps, Ls, bp_view_groups(Ps, w.geom.n_views))
+        fwd_bytes += fwd
+        bp_bytes += bp
     per_kernel = {}
     for name, ms, nbytes in (("proj", kms_default[0], fwd_bytes), ("bp", kms_default[2], bp_bytes)):
         gbps = nbytes / (ms * 1e-3) / 1e9
