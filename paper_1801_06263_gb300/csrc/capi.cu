@@ -1,5 +1,7 @@
 // C-ABI of the library (include/osscir.h): context creation, validation,
 // per-geometry tables, and the per-iteration CUDA graph.
+#include <unistd.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -58,6 +60,8 @@ void free_ctx(osscir_ctx* h) {
                     h->bp_slot, h->bp_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    if (h->report_locked) cudaHostUnregister(h->report);
+    std::free(h->report);
     delete h;
 }
 
@@ -287,6 +291,11 @@ osscir_status build(osscir_ctx* h, const osscir_geometry* g, const osscir_spectr
     CK(dalloc(&h->dtpl_part, h->n_part));
     CK(dalloc(&h->dtpl_out, 3));
     h->bad_counts = reinterpret_cast<int*>(h->dtpl_out + 2);
+    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    h->report = static_cast<osscir_ctx::Report*>(std::aligned_alloc(page, page));
+    if (!h->report) return OSSCIR_E_NOMEM;
+    h->report_locked = cudaHostRegister(h->report, page, cudaHostRegisterDefault) == cudaSuccess;
+    if (!h->report_locked) cudaGetLastError();   // the copies then go through the driver's own buffer
     if (h->inner > 1) CK(dalloc(&h->model, (size_t)kModelStride * L));
     CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&h->side_stream, cudaStreamNonBlocking));
@@ -751,11 +760,10 @@ osscir_status osscir_reconstruct(osscir_t h, const float* c_host, int n_iters, f
         xs = h->xo;
     }
     CK(cudaMemcpyAsync(maps_out_host, xs, sizeof(float4) * h->P, cudaMemcpyDeviceToHost, st));
-    osscir_ctx::Report report;
-    CK(cudaMemcpyAsync(&report, h->dtpl_out, sizeof report, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->report, h->dtpl_out, sizeof *h->report, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     // D_TPL at the last expansion point (the value the iterations computed)
-    if (n_iters > 0 && !std::isfinite(report.dtpl[1])) return OSSCIR_E_DIVERGED;
+    if (n_iters > 0 && !std::isfinite(h->report->dtpl[1])) return OSSCIR_E_DIVERGED;
     return OSSCIR_OK;
 }
 
@@ -803,11 +811,10 @@ osscir_status osscir_dtpl(osscir_t h, int which, double* out, void* stream) {
         CK(launch_counts(h->gc, h->exc(), h->rec, h->spec(), h->x, nullptr, h->c, h->dtpl_part, st));
         CK(launch_dtpl_reduce(h->dtpl_part, h->n_part, h->dtpl_out, st));
     }
-    osscir_ctx::Report report;
-    CK(cudaMemcpyAsync(&report, h->dtpl_out, sizeof report, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->report, h->dtpl_out, sizeof *h->report, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    *out = report.dtpl[which];
-    if (report.bad) return OSSCIR_E_INVALID;
+    *out = h->report->dtpl[which];
+    if (h->report->bad) return OSSCIR_E_INVALID;
     if (!std::isfinite(*out)) return OSSCIR_E_DIVERGED;
     return OSSCIR_OK;
 }

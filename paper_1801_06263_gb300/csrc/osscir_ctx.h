@@ -44,13 +44,17 @@ struct osscir_ctx {
     double* dtpl_part = nullptr;
     double* dtpl_out = nullptr;   // [0]: at x (on request), [1]: at the last expansion point; bad_counts follows
     int* bad_counts = nullptr;    // (in the same allocation) set by the check of the counts osscir_set_counts loads (0: valid)
-    // dtpl_out and bad_counts as the host reads them, with one copy: two held the host twice
-    // (osscir_dtpl 24 -> 15 us).  A page-locked record is read 1 us faster and costs every
-    // context 310 us to make and release (64 x 64: 870 us created and closed, 560 without).
+    // dtpl_out and bad_counts as the host reads them, with one copy (two held the host
+    // twice: osscir_dtpl 24 -> 14 us) into a page of the heap that is locked for it where
+    // that is possible.  Locking it costs a context 50 us in all and saves 2 us a step and
+    // read-back against an unlocked record; cudaMallocHost and its release took 290 us in a
+    // process without other page-locked memory (64 x 64 created and closed 840 us, 600 now).
     struct Report {
         double dtpl[2];
         int bad;
     };
+    Report* report = nullptr;
+    bool report_locked = false;
     int n_part = 0;
     int exp_model = 0;   // counts model: 0 softexp (Eq. finalModel), 1 exp (Eq. fullModel)
     int iter = 0;
