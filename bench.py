@@ -73,14 +73,14 @@ FP32_LANES_PER_SM, SCHEDULERS_PER_SM, L1_BYTES_PER_CLK_PER_SM, L1_WAVEFRONTS_PER
 # elapsed SM cycles x the capturing GPU's SMs).  Valid only for that workload and for
 # the kernel sources they were taken on (source_sha, see _source_sha).
 NCU_WORKLOAD = "medium_256"
-_SHA = "dea47b757b48fa99"
+_SHA = "845581104ad5b147"
 NCU_COUNTS = {
-    "k_fp_proj": {"dram_bytes": 353642496 + 5072640, "warp_instructions": 15558048,
+    "k_fp_proj": {"dram_bytes": 353640448 + 5152768, "warp_instructions": 15558048,
                   "l1_wavefronts": 16744000, "source_sha": _SHA},
-    "k_mocca_ray": {"dram_bytes": 14810112 + 382208, "warp_instructions": 91877016,
+    "k_mocca_ray": {"dram_bytes": 14809088 + 346624, "warp_instructions": 91877016,
                     "l1_wavefronts": 8824000, "source_sha": _SHA},
     # the back-projection's two launches: k_fpb_bp and k_fpb_finish
-    "k_fpb_bp": {"dram_bytes": 459161344 + 9107200 + 19988992, "warp_instructions": 72630248 + 2023424,
+    "k_fpb_bp": {"dram_bytes": 459163136 + 9099520 + 19988992, "warp_instructions": 72630248 + 2041856,
                  "l1_wavefronts": 21878000 + 292000, "source_sha": _SHA},
 }
 
